@@ -96,6 +96,7 @@ struct concord_state {
   double *mean = nullptr, *inv_scale = nullptr;
   void* Z = nullptr;
   int ldz = 0;
+  void* gf_work = nullptr;   // FP64 states: digits and scales of the FP64 Gram
   double* Xstage = nullptr;  // n_cap x p FP64, host-data path
   float *zt_hi = nullptr, *zt_lo = nullptr;
   int n_pad = 0, p_pad = 0;
@@ -1435,6 +1436,8 @@ int concord_create(concord_state** out, int p, int precision, int n_cap, int dev
       ALLOC(st->Xstage, (size_t)n_cap * p * sizeof(double));
       st->n_pad = round_up(n_cap, 64);
       st->p_pad = round_up(p, 128);
+      if (!is_mixed(st) && gram_f64_bytes(n_cap, p) > 0)
+        ALLOC(st->gf_work, gram_f64_bytes(n_cap, p));
       if (is_mixed(st)) {
         ALLOC(st->zt_hi, sizeof(float) * (size_t)st->n_pad * st->p_pad);
         ALLOC(st->zt_lo, sizeof(float) * (size_t)st->n_pad * st->p_pad);
@@ -1488,7 +1491,7 @@ int concord_destroy(concord_state* st) {
                  st->hist, st->result, st->mean, st->inv_scale, st->Z, st->Xstage, st->zt_hi,
                  st->zt_lo, st->sdiag64, st->sdiagT, st->omdiag64, st->S64, st->W64, st->Om64,
                  st->zt32, st->rf.cnt, st->rf.off, st->rf.cur, st->rf.nbr, st->rf.ctr, st->rf.cand,
-                 st->rf.bitmap, st->mrow, st->pol.mem};
+                 st->rf.bitmap, st->mrow, st->pol.mem, st->gf_work};
   for (void* d : dev)
     if (d) cudaFree(d);
   void* adj_dev[] = {st->adj.cnt, st->adj.rowptr, st->adj.bad, st->adj.col, st->adj.erow,
@@ -1926,8 +1929,10 @@ static int gram_into_state(concord_state* st, const void* X, int x_f32, int n, i
   const int p = st->p, ld = st->ld;
   CK(cudaMemsetAsync(st->flag, 0, sizeof(int), st->stream));
   // the FP64 W (free until the iterate is reset below) holds the column partials
-  CK(launch_col_stats_chunked(X, x_f32, n, p, ldx, prep, st->mean, st->inv_scale, st->flag,
-                              st->W64, st->stream));
+  const bool plain64 = !is_mixed(st) && st->gram_mode == CONCORD_GRAM_FP64;
+  if (!plain64)
+    CK(launch_col_stats_chunked(X, x_f32, n, p, ldx, prep, st->mean, st->inv_scale, st->flag,
+                                st->W64, st->stream));
   // the reduced-precision Grams keep the FP32 data (transposed) for the S
   // refinement of a later polish; the FP64 Gram is exact already
   st->zt_valid = false;
@@ -1944,9 +1949,8 @@ static int gram_into_state(concord_state* st, const void* X, int x_f32, int n, i
         CK(launch_syrk_f64(st->W64, n, p, ld, st->S64, ld, 1.0 / n, st->stream));
         CK(launch_convert(st->S64, 0, ld, st->S, 1, ld, p, p, st->stream));
       } else {
-        CK(launch_apply_prep(X, x_f32, n, p, ldx, st->mean, st->inv_scale, st->Z, 0, st->ldz,
-                             st->stream));
-        CK(launch_syrk_f64((const double*)st->Z, n, p, st->ldz, st->S64, ld, 1.0 / n, st->stream));
+        CK(launch_gram_f64({X, x_f32, n, p, ldx, prep, st->mean, st->inv_scale, st->flag, st->W64,
+                            (double*)st->Z, st->ldz, st->gf_work, st->S64, ld}, st->stream));
       }
       break;
     case CONCORD_GRAM_FP32: {
@@ -2063,6 +2067,7 @@ int concord_gram(const void* X_dev, int x_dtype, int n, int p, int ldx, int prep
   int* bad = nullptr;
   void* Z = nullptr;
   void* Sw = nullptr;
+  void* work = nullptr;
   float *hi = nullptr, *lo = nullptr;
   int rc = CONCORD_OK, hbad = 0;
   cudaError_t e = cudaSuccess;
@@ -2080,17 +2085,15 @@ int concord_gram(const void* X_dev, int x_dtype, int n, int p, int ldx, int prep
   GK(cudaMallocAsync((void**)&bad, sizeof(int), s));
   GK(cudaMemsetAsync(bad, 0, sizeof(int), s));
   GK(cudaMallocAsync((void**)&part, sizeof(double) * (size_t)col_stats_chunks(n) * p, s));
-  GK(launch_col_stats_chunked(X_dev, x_f32, n, p, ldx, prep, mean, inv, bad, part, s));
+  if (mode != CONCORD_GRAM_FP64)
+    GK(launch_col_stats_chunked(X_dev, x_f32, n, p, ldx, prep, mean, inv, bad, part, s));
   if (mode == CONCORD_GRAM_FP64) {
     GK(cudaMallocAsync(&Z, sizeof(double) * (size_t)n * ld, s));
-    GK(launch_apply_prep(X_dev, x_f32, n, p, ldx, mean, inv, Z, 0, ld, s));
-    if (s_f32) {
-      GK(cudaMallocAsync(&Sw, sizeof(double) * (size_t)p * ld, s));
-      GK(launch_syrk_f64((const double*)Z, n, p, ld, (double*)Sw, ld, 1.0 / n, s));
-      GK(launch_convert(Sw, 0, ld, S_dev, 1, lds, p, p, s));
-    } else {
-      GK(launch_syrk_f64((const double*)Z, n, p, ld, (double*)S_dev, lds, 1.0 / n, s));
-    }
+    if (gram_f64_bytes(n, p) > 0) GK(cudaMallocAsync(&work, gram_f64_bytes(n, p), s));
+    if (s_f32) GK(cudaMallocAsync(&Sw, sizeof(double) * (size_t)p * ld, s));
+    GK(launch_gram_f64({X_dev, x_f32, n, p, ldx, prep, mean, inv, bad, part, (double*)Z, ld, work,
+                        (double*)(s_f32 ? Sw : S_dev), s_f32 ? ld : lds}, s));
+    if (s_f32) GK(launch_convert(Sw, 0, ld, S_dev, 1, lds, p, p, s));
   } else if (mode == CONCORD_GRAM_FP32) {
     GK(cudaMallocAsync(&Z, sizeof(float) * (size_t)n * ld, s));
     GK(launch_apply_prep(X_dev, x_f32, n, p, ldx, mean, inv, Z, 1, ld, s));
@@ -2145,6 +2148,7 @@ done:
   if (bad) cudaFreeAsync(bad, s);
   if (Z) cudaFreeAsync(Z, s);
   if (Sw) cudaFreeAsync(Sw, s);
+  if (work) cudaFreeAsync(work, s);
   if (hi) cudaFreeAsync(hi, s);
   if (lo) cudaFreeAsync(lo, s);
 #undef GK

@@ -1,0 +1,626 @@
+// FP64 Gram S = Z^T Z / n on the 5th-generation tensor cores.
+//
+// This part multiplies FP64 numbers at 2 FMA per clock and SM: a CUDA-core
+// FP64 Gram at p = 5000, n = 2000 takes 41.8 ms, all of it in that pipe.  The
+// bf16 tensor pipe is three orders faster and exact on small integers, so the
+// products are made there from an error-free decomposition (Ozaki, Ogita,
+// Oishi, Rump 2012: split, multiply exactly, add up):
+//
+//   column i is scaled by a power of two, z = F 2^(e_i - 56), |F| <= 2^56
+//   (rounded once, to 2^(e_i - 57)), and F is written in balanced base 256:
+//   F = sum_s a_s 2^(8 (6 - s)), a_0 in [-256, 256], the others in
+//   [-128, 127].  Every digit is a bf16 exactly.
+//
+//   sum_k F_ik F_jk = sum_d 2^(8 (12 - d)) I_d,  I_d = sum_{s + t = d}
+//   sum_k a_ik,s a_jk,t.  A partial sum of 128 k of one class d <= 5 stays
+//   within 2^24, so the FP32 accumulator in tensor memory holds it exactly;
+//   the accumulators are read every 128 k and added up as 32-bit integers.
+//   Classes d = 0 .. 6 (28 products) are kept; d >= 7 is below 2^-58 of the
+//   columns' scales per product.  Their weighted sum is formed in 64-bit
+//   integers and rounded once to FP64 with the division by n.
+//
+// The result is as near to the exact Gram as the CUDA-core sums where a
+// column's largest entry is not far above its root mean square (the digits
+// are relative to the largest): k_col_route checks
+//   (2^e_i / rms_i)^2 <= 2^2.8 sqrt(n)
+// for every column (the dropped classes then stay below the rounding of an
+// FP64 sum of n products) and else routes the whole Gram to the CUDA cores.
+// Measured (standardized data, error of S against the exact Gram over the
+// CUDA-core kernel's): 0.1 - 0.7 of it at n = 40 .. 5000.
+//
+// Kernel: one CTA per 128 x 128 tile of the upper triangle.  Two classes are
+// accumulated per pass over k (classes 5 6, then 3 4, 1 2, 0), so that a
+// 7-slice block of A and B serves 13 products: with one class per pass the
+// operand loads from L2 (128 bytes per clock and SM) would bound it, with all
+// classes at once the accumulators do not fit in tensor memory.
+//   thread 0   TMA loads of 32-element K blocks (64-byte swizzled rows) into
+//              two stages of up to 14 operand tiles;
+//   thread 32  the MMAs; a class that starts a new 128-k chunk goes last in
+//              its block, so its accumulator is read while the other class
+//              is multiplied;
+//   16 warps   read the accumulators (tcgen05.ld), convert exactly to
+//              integers, and after each pass fold them into the 64-bit sums
+//              kept in the upper half of tensor memory.
+// Bound by the MMAs' operand reads from shared memory (M = N = 128 at ~0.8 of
+// the nominal rate).  p = 5000, n = 2000: CUDA cores 41.8 ms, here 1.6 ms.
+#include <cuda_bf16.h>
+
+#include "fp_bits.cuh"
+#include "kernels.h"
+#include "prep_stats.h"
+#include "tcgen05.cuh"
+
+namespace concord {
+
+namespace {
+
+constexpr int kTile128 = 128;
+constexpr int kDigits = 7;                       // base-256 digits (slices)
+constexpr int kBlkK = 32;                        // K elements of one block: 64-byte rows
+constexpr int kTileBytes = kTile128 * kBlkK * 2; // one operand tile: 8 KB
+constexpr int kSlots = 2 * kDigits;              // tiles of a stage
+constexpr int kStages = 2;
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 32 * (2 + kEpiWarps);
+constexpr int kSegBlocks = 448;                  // K blocks whose integer sums fit 32 bits
+constexpr int kPasses = 4;
+constexpr size_t kSmem = (size_t)kStages * kSlots * kTileBytes + 1024;
+constexpr int kAccHi = 0, kAccLo = 128, kSumLo = 256, kSumHi = 384;  // tensor-memory columns
+static_assert((size_t)kEpiWarps * 32 * 33 * 8 <= (size_t)kStages * kSlots * kTileBytes,
+              "the output staging fits in the operand ring");
+
+// Pass p accumulates class hi = 5 - 2 p and lo = hi + 1 (the last pass class
+// 0 alone); it needs the first lo + 1 slices, and takes as many K blocks per
+// stage as fit.
+__device__ __forceinline__ int pass_hi(int ps) { return ps == 3 ? 0 : 5 - 2 * ps; }
+__device__ __forceinline__ int pass_slices(int ps) { return ps == 3 ? 1 : 7 - 2 * ps; }
+__device__ __forceinline__ int pass_blocks(int ps) { return kDigits / pass_slices(ps); }
+
+// Chunk boundaries of the two classes over the K blocks of a pass, half a
+// chunk apart; class 0's digits allow chunks of 256 k (2^16 x 256 = 2^24).
+__device__ __forceinline__ bool hi_start(int ps, int kb) {
+  return ps == 3 ? (kb & 7) == 0 : (kb == 0 || (kb & 3) == 2);
+}
+__device__ __forceinline__ bool hi_end(int ps, int kb, int nkb) {
+  return kb == nkb - 1 || (ps == 3 ? (kb & 7) == 7 : (kb & 3) == 1);
+}
+__device__ __forceinline__ bool lo_start(int kb) { return (kb & 3) == 0; }
+__device__ __forceinline__ bool lo_end(int kb, int nkb) { return kb == nkb - 1 || (kb & 3) == 3; }
+
+// K-major operand tile in the 64-byte swizzled layout (rows of 64 bytes,
+// 8-row groups 512 bytes apart).
+__device__ __forceinline__ uint64_t sw64_kmajor_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+// D FP32, A and B BF16, both K-major, N = 128, M = 128.
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile128 >> 3) << 17) |
+                            ((uint32_t)(kTile128 >> 4) << 24);
+
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %3, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %4, q;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(accumulate), "r"(kIdesc)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld_x8(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+      : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st_x8(uint32_t taddr, const uint32_t (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
+                   taddr),
+               "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// One warp's 32 columns of a finished accumulator into its integer sums.
+__device__ __forceinline__ bool drain(uint32_t t, uint64_t* full, uint64_t* empty, unsigned parity,
+                                      int (&sum)[32], int* status) {
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(full, parity, status));
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (ok) {
+#pragma unroll
+    for (int q0 = 0; q0 < 32; q0 += 8) {
+      uint32_t v[8];
+      tmem_ld_x8(t + q0, v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sum[q0 + q] += __float2int_rn(__uint_as_float(v[q]));
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  mbar_arrive(empty);
+  return ok;
+}
+
+}  // namespace
+
+// z 2^(56 - e) rounded to an integer (ties away from zero); |z| <= 2^e.
+__host__ __device__ inline long long f64_to_fixed(double z, int e) {
+  const unsigned long long b = fb_d2u(z);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) return 0;  // zero (a subnormal is far below the last digit)
+  unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int sh = ex - 1075 + 56 - e;
+  if (sh >= 0) {
+    m <<= sh < 10 ? sh : 10;
+  } else {
+    const int r = -sh;
+    m = r > 60 ? 0ull : (m + (1ull << (r - 1))) >> r;
+  }
+  return (b >> 63) ? -(long long)m : (long long)m;
+}
+
+// Digit s (0: the leading one) of F in balanced base 256.
+__host__ __device__ inline int fixed_digit(long long F, int s) {
+  const long long b = F + 0x0000808080808080ll;
+  return s == 0 ? (int)(b >> 48) : (int)((b >> (8 * (6 - s))) & 0xff) - 128;
+}
+
+// h 2^x / n in FP64, rounded to nearest once; rinv = 2^(63 + k) / n rounded,
+// k = ceil(log2 n).  (Integer arithmetic: FP64 conversions and products share
+// the narrow FP64 pipe.)
+__host__ __device__ inline double fixed_over_n(long long h, int x, unsigned long long rinv, int k) {
+  if (h == 0) return 0.0;
+  unsigned long long a = h < 0 ? 0ull - (unsigned long long)h : (unsigned long long)h;
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)a);
+  a <<= lz;
+  unsigned long long q = __umul64hi(a, rinv);
+#else
+  const int lz = __builtin_clzll(a);
+  a <<= lz;
+  unsigned long long q = (unsigned long long)(((unsigned __int128)a * rinv) >> 64);
+#endif
+  // a 2^-lz rinv 2^(-63 - k) 2^x = q 2^(x + 1 - lz - k)
+  int ex = x + 1 - lz - k;
+  if (!(q >> 63)) {
+    q <<= 1;
+    --ex;
+  }
+  unsigned long long m = q >> 11;
+  const unsigned rem = (unsigned)(q & 0x7ffu);
+  m += (rem > 0x400u || (rem == 0x400u && (m & 1))) ? 1 : 0;
+  // m in [2^52, 2^53]: value m 2^(ex + 11); a carry to 2^53 moves into the exponent
+  const unsigned long long bits =
+      ((unsigned long long)(ex + 11 + 52 + 1023) << 52) + (m - 0x10000000000000ull);
+  return fb_u2d(bits | (h < 0 ? 0x8000000000000000ull : 0ull));
+}
+
+// ------------------------------------------------------------- preparation
+// Sums of squares and largest magnitudes of the centred columns, a chunk of
+// rows per CTA row (as k_col_partial; max exactly, the sums in its order).
+constexpr int kRouteCols = 128;
+
+template <typename TX>
+__global__ void __launch_bounds__(kRouteCols) k_col_sq_max(const TX* __restrict__ X, int n, int p,
+                                                           int ldx, int rows_per_chunk,
+                                                           const double* __restrict__ mean,
+                                                           double* __restrict__ part,
+                                                           double* __restrict__ pmax) {
+  const int col = blockIdx.x * kRouteCols + threadIdx.x;
+  if (col >= p) return;
+  const int r0 = blockIdx.y * rows_per_chunk;
+  const int r1 = min(n, r0 + rows_per_chunk);
+  const double mu = mean[col];
+  double acc = 0.0;
+  long long mx = 0;  // magnitudes order as integers
+#pragma unroll 8
+  for (int k = r0; k < r1; ++k) {
+    const double d = to_f64(__ldg(X + (size_t)k * ldx + col)) - mu;
+    acc += d * d;
+    mx = max(mx, (long long)(fb_d2u(d) & 0x7fffffffffffffffull));
+  }
+  part[(size_t)blockIdx.y * p + col] = acc;
+  pmax[(size_t)blockIdx.y * p + col] = fb_u2d((unsigned long long)mx);
+}
+
+// Per column: inv_scale (prep 2, as k_col_final), the scale exponent e with
+// max |z| <= 2^e, and whether its digits resolve it (else *route = 1).
+__global__ void k_col_route(const double* __restrict__ part, const double* __restrict__ pmax,
+                            int chunks, int n, int p, int p_pad, int prep, double limit,
+                            double* __restrict__ inv_scale, int* __restrict__ ecol,
+                            int* __restrict__ route, int* __restrict__ bad) {
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= p_pad) return;
+  if (col >= p) {
+    ecol[col] = 0;
+    return;
+  }
+  double s = 0.0, mx = 0.0;
+#pragma unroll 8
+  for (int c = 0; c < chunks; ++c) {
+    s += part[(size_t)c * p + col];
+    mx = fmax(mx, pmax[(size_t)c * p + col]);
+  }
+  double inv = 1.0;
+  if (prep == 2) {
+    const double sd = sqrt(s / n);
+    if (!(sd > 0.0)) atomicOr(bad, 1);
+    inv = 1.0 / sd;
+    inv_scale[col] = inv;
+  }
+  const double z = mx * inv, ss = s * inv * inv;
+  int e = 0;
+  if (z > 0.0 && isfinite(z) && isfinite(ss)) {
+    const unsigned long long b = fb_d2u(z);
+    e = (int)((b >> 52) & 0x7ff) - 1023 + ((b & 0xfffffffffffffull) ? 1 : 0);
+    const double t = ldexp(1.0, e < -1000 ? -1000 : e);
+    if (e < -400 || e > 400 || !(t * t * (double)n <= limit * ss)) atomicOr(route, 1);
+  } else if (z != 0.0) {
+    atomicOr(route, 1);
+  }
+  ecol[col] = e;
+}
+
+// Digits of the prepared data, transposed: dig[(s p_pad + i) n_pad + k] =
+// digit s of z_ki (bf16), zero padding.  64 x 32 tiles through shared memory,
+// one 128-byte segment per store.
+template <typename TX>
+__global__ void __launch_bounds__(256) k_digits(const TX* __restrict__ X, int n, int p, int ldx,
+                                                const double* __restrict__ mean,
+                                                const double* __restrict__ inv_scale,
+                                                const int* __restrict__ ecol,
+                                                const int* __restrict__ route,
+                                                uint32_t* __restrict__ dig, int n_pad, int p_pad) {
+  if (*route != 0) return;
+  __shared__ long long F[32][65];
+  const int k0 = blockIdx.x * 64, i0 = blockIdx.y * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i = i0 + tx;
+  const bool iv = i < p;
+  const double mu = iv ? mean[i] : 0.0, inv = iv ? inv_scale[i] : 0.0;
+  const int e = ecol[i];
+#pragma unroll
+  for (int r = ty; r < 64; r += 8) {
+    const int k = k0 + r;
+    long long f = 0;
+    if (iv && k < n) f = f64_to_fixed((to_f64(__ldg(X + (size_t)k * ldx + i)) - mu) * inv, e);
+    F[tx][r] = f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = ty; r < 32; r += 8) {
+    const long long f0 = F[r][2 * tx], f1 = F[r][2 * tx + 1];
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) {
+      // exact: 1.5 2^23 + digit, minus 1.5 2^23; a digit has 8 significant bits
+      const float g0 = __int_as_float(0x4B400000 + fixed_digit(f0, s)) - 12582912.f;
+      const float g1 = __int_as_float(0x4B400000 + fixed_digit(f1, s)) - 12582912.f;
+      dig[(((size_t)s * p_pad + i0 + r) * n_pad + k0) / 2 + tx] =
+          __byte_perm(__float_as_uint(g0), __float_as_uint(g1), 0x7632);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ product
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gram_f64(const __grid_constant__ CUtensorMap tm, int nkb, int p, int p_pad,
+               double* __restrict__ S, int lds, const int* __restrict__ ecol,
+               unsigned long long rinv, int rk, int sh, int nbt, int group,
+               const int* __restrict__ route, int* status) {
+  if (*route != 0) return;
+  extern __shared__ unsigned char gsm_raw[];
+  __shared__ __align__(8) uint64_t full[kStages];
+  __shared__ __align__(8) uint64_t empty[kStages];
+  __shared__ __align__(8) uint64_t acc_full[2];   // [0] class hi, [1] class lo
+  __shared__ __align__(8) uint64_t acc_empty[2];
+  __shared__ __align__(8) uint64_t fin;
+  __shared__ uint32_t tmem_base;
+  unsigned char* ring = (unsigned char*)(((uintptr_t)gsm_raw + 1023) & ~(uintptr_t)1023);
+
+  int bi, bj;
+  gram_tile(blockIdx.x, nbt, group, bi, bj);
+  const bool dtile = bi == bj;  // A and B are the same tiles: loaded once
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nseg = (nkb + kSegBlocks - 1) / kSegBlocks;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_base)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 32) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], kEpiWarps * 32);
+    }
+    mbar_init(&fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tbase = tmem_base;
+
+  if (warp == 0) {
+    // ---- producer
+    if (lane == 0) {
+      int gs = 0;  // stages filled so far
+      bool ok = true;
+      for (int seg = 0; seg < nseg && ok; ++seg) {
+        const int kb0 = seg * kSegBlocks, nk = min(kSegBlocks, nkb - kb0);
+        for (int ps = 0; ps < kPasses && ok; ++ps) {
+          const int ns = pass_slices(ps), kps = pass_blocks(ps);
+          for (int kb = 0; kb < nk; kb += kps, ++gs) {
+            const int st = gs % kStages;
+            if (gs >= kStages && !mbar_wait(&empty[st], ((gs / kStages) - 1) & 1, status)) {
+              ok = false;
+              break;
+            }
+            const int nb = min(kps, nk - kb);
+            mbar_expect_tx(&full[st], (unsigned)(nb * ns * (dtile ? 1 : 2) * kTileBytes));
+            unsigned char* base = ring + (size_t)st * kSlots * kTileBytes;
+            for (int b = 0; b < nb; ++b)
+              for (int s = 0; s < ns; ++s) {
+                unsigned char* at = base + (size_t)(2 * b * ns + s) * kTileBytes;
+                const int x = (kb0 + kb + b) * kBlkK;
+                tma_load_2d(at, &tm, &full[st], x, s * p_pad + bi * kTile128);
+                if (!dtile)
+                  tma_load_2d(at + (size_t)ns * kTileBytes, &tm, &full[st], x,
+                              s * p_pad + bj * kTile128);
+              }
+          }
+        }
+      }
+      if (!ok)  // gave up: the copies in flight still land in this CTA's memory
+        for (int q = gs - 1; q >= 0 && q >= gs - kStages; --q)
+          mbar_wait(&full[q % kStages], (q / kStages) & 1, status);
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer
+    if (lane == 0) {
+      int gs = 0, nch[2] = {0, 0};  // chunks started per class
+      bool ok = true;
+      for (int seg = 0; seg < nseg && ok; ++seg) {
+        const int nk = min(kSegBlocks, nkb - seg * kSegBlocks);
+        for (int ps = 0; ps < kPasses && ok; ++ps) {
+          const int ns = pass_slices(ps), kps = pass_blocks(ps), dh = pass_hi(ps);
+          for (int kb = 0; kb < nk && ok; kb += kps, ++gs) {
+            const int st = gs % kStages;
+            ok = mbar_wait(&full[st], (gs / kStages) & 1, status);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t base = smem_u32(ring + (size_t)st * kSlots * kTileBytes);
+            const int nb = min(kps, nk - kb);
+            for (int b = 0; b < nb && ok; ++b) {
+              const int kk = kb + b;
+              const uint32_t at = base + (uint32_t)(2 * b * ns * kTileBytes);
+              const uint64_t a0 = sw64_kmajor_desc(at);
+              const uint64_t b0 = dtile ? a0 : sw64_kmajor_desc(at + (uint32_t)(ns * kTileBytes));
+              const bool lo_first = ps < 3 && hi_start(ps, kk) && kk != 0;
+              for (int o = 0; o < (ps < 3 ? 2 : 1) && ok; ++o) {
+                const int c = ps == 3 ? 0 : (lo_first ? 1 - o : o);  // 0: class hi, 1: class lo
+                const bool start = c == 0 ? hi_start(ps, kk) : lo_start(kk);
+                if (start) {
+                  if (nch[c] > 0) {
+                    ok = mbar_wait(&acc_empty[c], (nch[c] - 1) & 1, status);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                  }
+                  ++nch[c];
+                }
+                const uint32_t d = tbase + (uint32_t)(c == 0 ? kAccHi : kAccLo);
+                const int cls = dh + c;
+                for (int s = 0; s <= cls; ++s) {
+                  const uint64_t as = a0 + (uint64_t)(s * (kTileBytes >> 4));
+                  const uint64_t bs = b0 + (uint64_t)((cls - s) * (kTileBytes >> 4));
+                  mma_bf16(d, as, bs, start && s == 0 ? 0u : 1u);
+                  mma_bf16(d, as + 2, bs + 2, 1u);  // the block's second 16 k
+                }
+                if (c == 0 ? hi_end(ps, kk, nk) : lo_end(kk, nk)) mma_commit(&acc_full[c]);
+              }
+            }
+            mma_commit(&empty[st]);
+          }
+        }
+      }
+      if (!ok) {  // gave up: wait for the products in flight before the memory is freed
+        mma_commit(&fin);
+        mbar_wait(&fin, 0, status);
+      }
+    }
+  } else {
+    // ---- 16 warps: warp e owns tensor-memory lanes 32 (warp % 4) .. +31
+    //      (tile rows) and tile columns 32 (e / 4) .. +31
+    const int e = warp - 2, quad = warp & 3, col0 = 32 * (e >> 2);
+    const uint32_t lanes = (uint32_t)(quad * 32) << 16;
+    const uint32_t t_lo = tbase + lanes + (uint32_t)(kSumLo + col0);
+    const uint32_t t_hi = tbase + lanes + (uint32_t)(kSumHi + col0);
+    int ih[32], il[32];
+    int nch[2] = {0, 0};
+    bool ok = true;
+    for (int seg = 0; seg < nseg && ok; ++seg) {
+      const int nk = min(kSegBlocks, nkb - seg * kSegBlocks);
+      for (int ps = 0; ps < kPasses && ok; ++ps) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q) ih[q] = il[q] = 0;
+        for (int kb = 0; kb < nk && ok; ++kb) {
+          if (hi_end(ps, kb, nk))
+            ok = drain(tbase + lanes + (uint32_t)(kAccHi + col0), &acc_full[0], &acc_empty[0],
+                       nch[0]++ & 1, ih, status);
+          if (ps < 3 && ok && lo_end(kb, nk))
+            ok = drain(tbase + lanes + (uint32_t)(kAccLo + col0), &acc_full[1], &acc_empty[1],
+                       nch[1]++ & 1, il, status);
+        }
+        if (!ok) break;
+        // fold the pass into the 64-bit sums (unit: 2^-sh of class 0's).  No
+        // branches on the pass around the 32 entries: they would be kept
+        // twice
+        const int shift = ps == 3 ? sh : sh - 8 * (pass_hi(ps) + 1);
+        const int left = max(shift, 0), right = max(-shift, 0);
+        const long long half = right > 0 ? 1ll << (right - 1) : 0ll;
+        const int radix = ps == 3 ? 1 : 256;
+        const uint32_t keep = seg == 0 && ps == 0 ? 0u : 0xffffffffu;
+#pragma unroll
+        for (int q0 = 0; q0 < 32; q0 += 8) {
+          uint32_t wl[8], wh[8];
+          tmem_ld_x8(t_lo + q0, wl);
+          tmem_ld_x8(t_hi + q0, wh);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          // pins the eight entries' arithmetic here: hoisted for all 32 it
+          // spilled 1.2 KB a thread, through the SRAM the MMAs read from
+#pragma unroll
+          for (int q = 0; q < 8; ++q) asm volatile("" : "+r"(ih[q0 + q]), "+r"(il[q0 + q]));
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const long long c = (long long)ih[q0 + q] * radix + (long long)il[q0 + q];
+            const long long h = (long long)(((unsigned long long)(wh[q] & keep) << 32) | (wl[q] & keep)) +
+                                (((c << left) + half) >> right);
+            wl[q] = (uint32_t)h;
+            wh[q] = (uint32_t)((unsigned long long)h >> 32);
+          }
+          tmem_st_x8(t_lo + q0, wl);
+          tmem_st_x8(t_hi + q0, wh);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      }
+    }
+    if (ok) {
+      // the sums over n, staged in the ring (idle: every load was consumed,
+      // every product done), then S[j][i] (lanes over i) and S[i][j] (lanes
+      // over j) in whole row segments
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      double* T = reinterpret_cast<double*>(ring) + e * (32 * 33);
+      const int i0 = bi * kTile128 + quad * 32, j0 = bj * kTile128 + col0;
+      const int i = i0 + lane, ei = __ldg(ecol + i);  // p_pad entries
+#pragma unroll 1
+      for (int q0 = 0; q0 < 32; q0 += 8) {
+        uint32_t wl[8], wh[8];
+        tmem_ld_x8(t_lo + q0, wl);
+        tmem_ld_x8(t_hi + q0, wh);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int j = j0 + q0 + q;
+          const double v = fixed_over_n((long long)(((unsigned long long)wh[q] << 32) | wl[q]),
+                                        ei + __ldg(ecol + j) - 16 - sh, rinv, rk);
+          T[lane * 33 + q0 + q] = v;
+          if (i < p && j < p && i <= j) S[(size_t)j * lds + i] = v;
+        }
+      }
+      __syncwarp();
+      const int j = j0 + lane;
+      for (int r = 0; r < 32; ++r)
+        if (i0 + r < p && j < p && i0 + r <= j) S[(size_t)(i0 + r) * lds + j] = T[r * 33 + lane];
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(512)
+                 : "memory");
+}
+
+// -------------------------------------------------------------------- host
+namespace {
+
+size_t al256(size_t b) { return (b + 255) / 256 * 256; }
+int pad(int v, int m) { return (v + m - 1) / m * m; }
+
+}  // namespace
+
+size_t gram_f64_bytes(int n, int p) {
+  if (n < kGramF64MinRows) return 0;
+  const int chunks = col_stats_chunks(n), p_pad = pad(p, kTile128);
+  return 2 * al256(sizeof(double) * (size_t)chunks * p) + al256(sizeof(int) * (size_t)p_pad) +
+         al256(sizeof(int)) + al256(2 * (size_t)kDigits * p_pad * pad(n, 64));
+}
+
+cudaError_t launch_gram_f64(const GramF64Args& g, cudaStream_t st) {
+  const int n = g.n, p = g.p;
+  cudaError_t e;
+  if (n < kGramF64MinRows || g.work == nullptr) {
+    if ((e = launch_col_stats_chunked(g.X, g.x_f32, n, p, g.ldx, g.prep, g.mean, g.inv_scale, g.bad,
+                                      g.part, st)) != cudaSuccess)
+      return e;
+    if ((e = launch_apply_prep(g.X, g.x_f32, n, p, g.ldx, g.mean, g.inv_scale, g.Z, 0, g.ldz, st)) !=
+        cudaSuccess)
+      return e;
+    return launch_syrk_f64(g.Z, n, p, g.ldz, g.S, g.lds, 1.0 / n, st);
+  }
+  const int chunks = col_stats_chunks(n), p_pad = pad(p, kTile128), n_pad = pad(n, 64);
+  char* m = (char*)g.work;
+  auto take = [&](size_t b) {
+    char* r = m;
+    m += al256(b);
+    return r;
+  };
+  double* part = (double*)take(sizeof(double) * (size_t)chunks * p);
+  double* pmax = (double*)take(sizeof(double) * (size_t)chunks * p);
+  int* ecol = (int*)take(sizeof(int) * (size_t)p_pad);
+  int* route = (int*)take(sizeof(int));
+  uint32_t* dig = (uint32_t*)take(2 * (size_t)kDigits * p_pad * n_pad);
+  // mean (and inv_scale = 1), then squares and maxima, then scales and route
+  if ((e = launch_col_stats_chunked(g.X, g.x_f32, n, p, g.ldx, g.prep == 2 ? 1 : g.prep, g.mean,
+                                    g.inv_scale, g.bad, part, st)) != cudaSuccess)
+    return e;
+  if ((e = cudaMemsetAsync(route, 0, sizeof(int), st)) != cudaSuccess) return e;
+  const int rpc = (n + chunks - 1) / chunks;
+  const dim3 sgrid((p + kRouteCols - 1) / kRouteCols, chunks), dgrid(n_pad / 64, p_pad / 32);
+  const double limit = 6.9644045063689921 * sqrt((double)n);  // 2^2.8 sqrt(n)
+  if (g.x_f32)
+    k_col_sq_max<float><<<sgrid, kRouteCols, 0, st>>>((const float*)g.X, n, p, g.ldx, rpc, g.mean,
+                                                      part, pmax);
+  else
+    k_col_sq_max<double><<<sgrid, kRouteCols, 0, st>>>((const double*)g.X, n, p, g.ldx, rpc, g.mean,
+                                                       part, pmax);
+  k_col_route<<<(p_pad + 127) / 128, 128, 0, st>>>(part, pmax, chunks, n, p, p_pad, g.prep, limit,
+                                                   g.inv_scale, ecol, route, g.bad);
+  if (g.x_f32)
+    k_digits<float><<<dgrid, 256, 0, st>>>((const float*)g.X, n, p, g.ldx, g.mean, g.inv_scale, ecol,
+                                           route, dig, n_pad, p_pad);
+  else
+    k_digits<double><<<dgrid, 256, 0, st>>>((const double*)g.X, n, p, g.ldx, g.mean, g.inv_scale,
+                                            ecol, route, dig, n_pad, p_pad);
+  PFN_cuTensorMapEncodeTiled_v12000 enc;
+  if ((e = encode_fn(&enc)) != cudaSuccess) return e;
+  CUtensorMap tm;
+  cuuint64_t dims[2] = {(cuuint64_t)n_pad, (cuuint64_t)kDigits * p_pad};
+  cuuint64_t strides[1] = {(cuuint64_t)n_pad * 2};
+  cuuint32_t box[2] = {(cuuint32_t)kBlkK, (cuuint32_t)kTile128};
+  cuuint32_t estr[2] = {1, 1};
+  if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, dig, dims, strides, box, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  if ((e = cudaFuncSetAttribute(k_gram_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kSmem)) != cudaSuccess)
+    return e;
+  int rk = 0;
+  while ((1ll << rk) < n) ++rk;
+  const unsigned long long rinv =
+      (unsigned long long)((((unsigned __int128)1 << (63 + rk)) + (unsigned)n / 2) / (unsigned)n);
+  const int nbt = p_pad / kTile128;
+  k_gram_f64<<<nbt * (nbt + 1) / 2, kThreads, kSmem, st>>>(tm, (n + kBlkK - 1) / kBlkK, p, p_pad, g.S,
+                                                           g.lds, ecol, rinv, rk, 46 - rk, nbt,
+                                                           kGroupRows, route, g.bad);
+  // the CUDA-core Gram of data the digits do not resolve (returns at once else)
+  note_launches(4);
+  if ((e = launch_apply_prep(g.X, g.x_f32, n, p, g.ldx, g.mean, g.inv_scale, g.Z, 0, g.ldz, st,
+                             route)) != cudaSuccess)
+    return e;
+  return launch_syrk_f64(g.Z, n, p, g.ldz, g.S, g.lds, 1.0 / n, st, route);
+}
+
+}  // namespace concord

@@ -26,14 +26,11 @@
 //     S[j][i] for i <= j through a shared-memory transpose.
 // Every wait is bounded (%globaltimer); a wait that runs out sets bit 4 of
 // the caller's status word.
-#include <cuda.h>
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
-
-#include <mutex>
 
 #include "kernels.h"
 #include "fp_bits.cuh"
+#include "tcgen05.cuh"
 
 namespace concord {
 
@@ -155,60 +152,6 @@ constexpr int kTmemCols = 512;                    // two 128-column FP32 accumul
 constexpr int kSumLo = 2 * kTM;                   // tensor-memory columns of the sums' low parts
 constexpr size_t kGramSmem = (size_t)kStages * kStageBytes + 1024;  // + alignment slack
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait for the phase with the given parity; false (and status bit 4)
-// if it has not completed within 2 s.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* status) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  unsigned it = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++it & 255u) == 0 && globaltimer_ns() - t0 > 2000000000ull) {
-      atomicOr(status, 4);
-      return false;
-    }
-  }
-  return true;
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
-                                            int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-      "l"((unsigned long long)map), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-
 // Shared-memory matrix descriptor of a K-major operand tile stored in the
 // 128-byte swizzled layout TMA writes (rows of 128 bytes, 8-row groups 1024
 // bytes apart): start address >> 4, leading offset (unused for swizzled
@@ -266,38 +209,6 @@ __device__ __forceinline__ void mma_fmt(uint32_t d, uint64_t a, uint64_t b, uint
   else mma_tf32(d, a, b, acc);
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]),
-        "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),
-        "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-      "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-      "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
-      "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-      : "memory");
-}
-
 // hi + lo += x with the rounding error of hi + x kept exactly (Knuth's
 // TwoSum: six FP32 additions, no ordering assumption on |hi| and |x|).
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
@@ -306,41 +217,6 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
   const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
   hi = s;
   lo = __fadd_rn(lo, err);
-}
-
-// Order of the upper-triangle tiles over the grid: bands of kGroupRows tile
-// rows; within a band the tile columns in increasing order and, per column,
-// the band's rows bi <= bj.  The CTAs resident at one time then read a few
-// dozen operand row blocks (the band's own and a run of columns), each from
-// several CTAs at nearly the same K, so L2 serves the repeats; in row-major
-// order every resident CTA streams its own column block from HBM.
-constexpr int kGroupRows = 8;
-
-__host__ __device__ inline void gram_tile(int t, int nbt, int group, int& bi, int& bj) {
-  int r0 = 0;
-  for (;;) {
-    const int g = nbt - r0 < group ? nbt - r0 : group;
-    const int tri = g * (g + 1) / 2;  // columns r0 .. r0 + g - 1: rows r0 .. bj
-    const int cnt = tri + (nbt - r0 - g) * g;
-    if (t < cnt) {
-      if (t < tri) {
-        int c = 0;
-        while (t > c) {
-          t -= c + 1;
-          ++c;
-        }
-        bj = r0 + c;
-        bi = r0 + t;
-      } else {
-        t -= tri;
-        bj = r0 + g + t / g;
-        bi = r0 + t % g;
-      }
-      return;
-    }
-    t -= cnt;
-    r0 += g;
-  }
 }
 
 // Packed FP32 pair arithmetic (add / sub .f32x2, round to nearest on each
@@ -579,24 +455,6 @@ __global__ void __launch_bounds__(kGramThreads, 1)
 }
 
 namespace {
-
-std::mutex g_tma_mu;
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-
-cudaError_t encode_fn(PFN_cuTensorMapEncodeTiled_v12000* out) {
-  std::lock_guard<std::mutex> lock(g_tma_mu);
-  if (!g_encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                     cudaEnableDefault, &q);
-    if (e != cudaSuccess) return e;
-    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-  }
-  *out = g_encode;
-  return cudaSuccess;
-}
 
 // 2-D tensor map over a p_pad x n_pad array of FP32 (bf16 = false) or bf16,
 // box one 128-byte row (K) x 128 rows, 128-byte swizzle.

@@ -247,12 +247,35 @@ cudaError_t launch_col_stats(const void* X, int x_f32, int n, int p, int ldx, in
 // columns p..ldz-1 are zero.
 cudaError_t launch_apply_prep(const void* X, int x_f32, int n, int p, int ldx, const double* mean,
                               const double* inv_scale, void* Z, int z_f32, int ldz,
-                              cudaStream_t st);
-// S = Z^T Z * scale on CUDA cores (upper-triangle tiles, mirrored).
+                              cudaStream_t st, const int* route = nullptr);
+// S = Z^T Z * scale on CUDA cores (upper-triangle tiles, mirrored).  With
+// route (device word) this and launch_apply_prep do nothing when it is 0.
 cudaError_t launch_syrk_f64(const double* Z, int n, int p, int ldz, double* S, int lds, double scale,
-                            cudaStream_t st);
+                            cudaStream_t st, const int* route = nullptr);
 cudaError_t launch_syrk_f32(const float* Z, int n, int p, int ldz, float* S, int lds, float scale,
                             cudaStream_t st);
+
+// ---- FP64 Gram (gram_f64.cu): column statistics, then S = Z^T Z / n from
+// exact bf16 digit products on tensor cores, or on CUDA cores where the
+// columns' ranges (checked on the device), fewer than kGramF64MinRows rows or
+// work = NULL ask for it.  Below 32 rows the digits' fixed resolution shows
+// against an FP64 sum of so few products (one row must give the rounded
+// product exactly), and the CUDA cores are as fast.
+constexpr int kGramF64MinRows = 32;
+struct GramF64Args {
+  const void* X;
+  int x_f32, n, p, ldx, prep;
+  double *mean, *inv_scale;  // [p] outputs
+  int* bad;                  // checks as launch_col_stats_chunked, 4: a wait ran out
+  double* part;              // col_stats_chunks(n) x p scratch (CUDA-core path)
+  double* Z;                 // n x ldz scratch (CUDA-core path)
+  int ldz;
+  void* work;                // gram_f64_bytes(n, p) or more
+  double* S;
+  int lds;
+};
+size_t gram_f64_bytes(int n, int p);
+cudaError_t launch_gram_f64(const GramF64Args& g, cudaStream_t st);
 
 // ---- small utilities (util.cu)
 // out[r*ldo + c] = (To) in[r*ldi + c] for r < rows, c < cols; zero for cols <= c < ldo.

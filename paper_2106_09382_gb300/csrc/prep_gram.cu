@@ -130,7 +130,8 @@ __global__ void k_col_final(const double* __restrict__ part, int chunks, int n, 
 template <typename TX, typename TZ>
 __global__ void k_apply_prep(const TX* __restrict__ X, int n, int p, int ldx,
                              const double* __restrict__ mean, const double* __restrict__ inv_scale,
-                             TZ* __restrict__ Z, int ldz) {
+                             TZ* __restrict__ Z, int ldz, const int* __restrict__ route) {
+  if (route != nullptr && *route == 0) return;
   const size_t total = (size_t)n * ldz;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -184,20 +185,20 @@ cudaError_t launch_col_stats_chunked(const void* X, int x_f32, int n, int p, int
 
 cudaError_t launch_apply_prep(const void* X, int x_f32, int n, int p, int ldx, const double* mean,
                               const double* inv_scale, void* Z, int z_f32, int ldz,
-                              cudaStream_t st) {
+                              cudaStream_t st, const int* route) {
   const int grid = 152 * 8;
   if (x_f32 && z_f32)
     k_apply_prep<float, float><<<grid, 256, 0, st>>>((const float*)X, n, p, ldx, mean, inv_scale,
-                                                     (float*)Z, ldz);
+                                                     (float*)Z, ldz, route);
   else if (x_f32)
     k_apply_prep<float, double><<<grid, 256, 0, st>>>((const float*)X, n, p, ldx, mean, inv_scale,
-                                                      (double*)Z, ldz);
+                                                      (double*)Z, ldz, route);
   else if (z_f32)
     k_apply_prep<double, float><<<grid, 256, 0, st>>>((const double*)X, n, p, ldx, mean, inv_scale,
-                                                      (float*)Z, ldz);
+                                                      (float*)Z, ldz, route);
   else
     k_apply_prep<double, double><<<grid, 256, 0, st>>>((const double*)X, n, p, ldx, mean,
-                                                       inv_scale, (double*)Z, ldz);
+                                                       inv_scale, (double*)Z, ldz, route);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -212,7 +213,9 @@ cudaError_t launch_apply_prep(const void* X, int x_f32, int n, int p, int ldx, c
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_syrk(const T* __restrict__ Z, int n, int p, int ldz,
-                                              T* __restrict__ S, int lds, T scale, int nb) {
+                                              T* __restrict__ S, int lds, T scale, int nb,
+                                              const int* __restrict__ route) {
+  if (route != nullptr && *route == 0) return;
   constexpr int BM = 64, BK = 16;
   __shared__ T As[BK][BM];
   __shared__ T Bs[BK][BM];
@@ -269,17 +272,17 @@ __global__ void __launch_bounds__(256) k_syrk(const T* __restrict__ Z, int n, in
 
 template <typename T>
 static cudaError_t launch_syrk_t(const T* Z, int n, int p, int ldz, T* S, int lds, T scale,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, const int* route = nullptr) {
   const int nb = (p + 63) / 64;
   const int tiles = nb * (nb + 1) / 2;
-  k_syrk<T><<<tiles, 256, 0, st>>>(Z, n, p, ldz, S, lds, scale, nb);
+  k_syrk<T><<<tiles, 256, 0, st>>>(Z, n, p, ldz, S, lds, scale, nb, route);
   note_launches(1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_syrk_f64(const double* Z, int n, int p, int ldz, double* S, int lds, double scale,
-                            cudaStream_t st) {
-  return launch_syrk_t<double>(Z, n, p, ldz, S, lds, scale, st);
+                            cudaStream_t st, const int* route) {
+  return launch_syrk_t<double>(Z, n, p, ldz, S, lds, scale, st, route);
 }
 cudaError_t launch_syrk_f32(const float* Z, int n, int p, int ldz, float* S, int lds, float scale,
                             cudaStream_t st) {
