@@ -46,7 +46,6 @@ constexpr int kMailboxDepth = kDepth;
 constexpr int kHistCap = 8192;
 constexpr int kMaxTimedLaunches = 16;
 constexpr int kDefaultPollNs = 0;
-
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 }  // namespace
@@ -383,7 +382,7 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
 // FP64 width, so both precisions fit) and one block holding the candidate
 // lists and per-candidate arrays, carved below.
 struct ScreenLayout {
-  size_t ctr, cand0, cand1, cnt_r0, cnt_r1, fail, off_r, cur_r, nd_pi, nd_pj, row_ent, term_ptr, term_pred, term_s, nd_rec, nd_delta, nd_new, nd_d2, jac,
+  size_t ctr, cand0, cand1, cnt_r0, cnt_r1, fail, off_r, cur_r, nd_pi, nd_pj, row_ent, term_ptr, term_pred, term_s, nd_rec, nd_delta, nd_new, jac,
       diag_old, omdiag_old, diag_new, dpart, dfill, diag_dd, pend_u, pend_d, pend_n, pend_new,
       rowacc, rowa_new, apart, loud, loudf, total;
 };
@@ -413,7 +412,6 @@ ScreenLayout screen_layout(int p, int P, int nc, int tc) {
   L.nd_rec = take(sizeof(double) * 4 * (size_t)nc);
   L.nd_delta = take(sizeof(double) * (size_t)nc);
   L.nd_new = take(sizeof(double) * (size_t)nc);
-  L.nd_d2 = take(sizeof(double) * (size_t)nc);
   L.jac = take(sizeof(unsigned long long) * kJacMax);
   L.diag_old = take(sizeof(double) * (size_t)p);
 
@@ -493,7 +491,6 @@ ScreenWork<T> screen_work(concord_state* st) {
   w.nd_rec = (T*)(b + L.nd_rec);
   w.nd_delta = (T*)(b + L.nd_delta);
   w.nd_new = (T*)(b + L.nd_new);
-  w.nd_d2 = (T*)(b + L.nd_d2);
   w.jac = (unsigned long long*)(b + L.jac);
   w.diag_old = (T*)(b + L.diag_old);
 

@@ -139,6 +139,7 @@ constexpr int kJacMax = 64;       // fixed-point iterations of the chain before 
 constexpr int kLoudMax = 256;     // rows a partial verification takes (more: a full sweep)
 constexpr int kStatusDense = 5;   // result status: the next sweep needs the dense kernel
 constexpr int kPendRow = 32;      // deferred W updates a row holds (lazy sweeps)
+constexpr int kMaxCluster = 16;   // CTAs of the largest thread-block cluster
 
 template <typename T>
 struct ScreenWork {
@@ -155,7 +156,6 @@ struct ScreenWork {
   T* term_s;                // [term_cap] the S entry it multiplies
   T* nd_rec;                // [4 nc_cap] per candidate: W_ij, W_ji, w_ij at the sweep start, s_ii + s_jj
   T *nd_delta, *nd_new;     // change and new value of each candidate
-  T* nd_d2;                 // [nc_cap] second buffer of the fixed-point iteration
   unsigned long long* jac;  // [kJacMax] per fixed-point round: arrivals + (CTAs whose changes moved) << 32
   T* diag_old;              // [p] diagonal before the sweep (for a redo)
   double* omdiag_old;       // [p] FP64 diagonal before the sweep (mixed precision)
@@ -228,10 +228,15 @@ struct ScreenArgs {
                             // host polishes it in FP64 and resumes the path after it)
 };
 
-size_t screened_dyn_smem(bool mixed);
 cudaError_t launch_screened(const ScreenArgs<double>& a, int grid, cudaStream_t st);
 cudaError_t launch_screened(const ScreenArgs<float>& a, int grid, cudaStream_t st);
 cudaError_t screened_occupancy(bool mixed, int* blocks_per_sm);
+// The same sweeps of n independent problems (a device table), their lambda
+// paths included, one thread-block cluster of `size` CTAs each (a power of
+// two up to screened_cluster_size(); 1: no cluster).
+cudaError_t launch_screened_batch(const ScreenArgs<double>* probs, int n, int size, cudaStream_t st);
+cudaError_t launch_screened_batch(const ScreenArgs<float>* probs, int n, int size, cudaStream_t st);
+cudaError_t screened_cluster_size(bool mixed, int* size);
 
 cudaError_t launch_refresh_w(const double* Om, const double* S, double* W, int p, int ld, int sms,
                              cudaStream_t st);

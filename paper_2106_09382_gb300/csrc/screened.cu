@@ -43,6 +43,15 @@ constexpr int kModeFull = 0, kModeLazy = 1, kModeDefer = 2, kModePartial = 3;
 // Candidates of one row sorted by a warp in shared memory (longer rows: one
 // thread, insertion sort).
 constexpr int kSortCap = 512;
+// Dynamic shared memory.  Per warp: the row pass's staged changes (partner,
+// step, delta), or the row sort's keys and steps; in the chain the owned
+// candidates' terms.
+__host__ __device__ constexpr size_t screened_dyn_smem(bool mixed) {
+  const size_t rows = (size_t)kRowList * (8 + (mixed ? 4 : 8));
+  const size_t sort = (size_t)2 * kSortCap * sizeof(int);
+  return (size_t)(kScreenThreads / 32) * (rows > sort ? rows : sort);
+}
+
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
@@ -66,6 +75,24 @@ struct Vec<double> {
   __device__ static void split(const V& v, double* o) { o[0] = v.x; o[1] = v.y; }
   __device__ static V join(const double* o) { return make_double2(o[0], o[1]); }
 };
+
+// Values other CTAs read while they change (single-copy atomic, through L2).
+__device__ __forceinline__ float ld_relaxed(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_relaxed(const double* p) {
+  double v;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(float* p, float v) {
+  asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed(double* p, double v) {
+  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
 
 __device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_uint(a) == __float_as_uint(b); }
 __device__ __forceinline__ bool same_bits(double a, double b) {
@@ -162,9 +189,9 @@ __device__ __forceinline__ void load8(const T* src, T (&o)[8]) {
   for (int q = 0; q < 8 / VT::N; ++q) VT::split(__ldcg(v + q), o + q * VT::N);
 }
 
-// Block reduction of the per-thread partials into partials[blockIdx.x*kParts+k].
+// Block reduction of the per-thread partials into partials[cta * kParts + k].
 __device__ __forceinline__ void reduce_parts(double (&v)[kParts], double* out,
-                                             double (*red)[kParts]) {
+                                             double (*red)[kParts], int cta) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < kParts; ++k) {
@@ -189,23 +216,22 @@ __device__ __forceinline__ void reduce_parts(double (&v)[kParts], double* out,
     if (lane == 0) red[wid][k] = x;
   }
   __syncthreads();
-  // the warps' values, part by part, over the lanes of warp 0 (a fixed tree;
-  // one thread adding them in turn was a chain of ~128 FP64 operations)
-  if (wid == 0) {
+  // the warps' values over the lanes of a warp, one part per warp (a fixed
+  // tree; one thread adding them in turn was a chain of ~128 FP64 operations)
+  static_assert(kParts <= kScreenThreads / 32, "a warp per part");
+  if (wid < kParts) {
+    const int k = wid;
+    double x = lane < nw ? red[lane][k] : 0.0;  // 0: the identity of both
+    if (k == kPartKkt || k == kPartDelta) {
+      long long m = __double_as_longlong(x);
 #pragma unroll
-    for (int k = 0; k < kParts; ++k) {
-      double x = lane < nw ? red[lane][k] : 0.0;  // 0: the identity of both
-      if (k == kPartKkt || k == kPartDelta) {
-        long long m = __double_as_longlong(x);
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(FULL, m, o));
+      x = __longlong_as_double(m);
+    } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(FULL, m, o));
-        x = __longlong_as_double(m);
-      } else {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(FULL, x, o);
-      }
-      if (lane == 0) out[(size_t)blockIdx.x * kParts + k] = x;
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(FULL, x, o);
     }
+    if (lane == 0) out[(size_t)cta * kParts + k] = x;
   }
   __syncthreads();
 }
@@ -336,6 +362,36 @@ __device__ __forceinline__ T pend_fold(const ScreenArgs<T>& a, int i, int n, int
       if (u[r] >= 0) wv = fma_t(d[r], sv[r], wv);
   }
   return wv;
+}
+
+// pend_fold of W_ij and W_ji together: the two rows' entries and S values are
+// requested at the same time.
+template <typename T>
+__device__ __forceinline__ void pend_fold2(const ScreenArgs<T>& a, int i, int j, int ni, int nj, T& wij,
+                                           T& wji) {
+  const int *pi = a.w.pend_u + (size_t)i * kPendRow, *pj = a.w.pend_u + (size_t)j * kPendRow;
+  const T *di = a.w.pend_d + (size_t)i * kPendRow, *dj = a.w.pend_d + (size_t)j * kPendRow;
+  for (int k0 = 0; k0 < max(ni, nj); k0 += 8) {
+    int u[8], v[8];
+    T du[8], dv[8], su[8], sv[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      u[r] = k0 + r < ni ? ldi(pi + k0 + r) : -1;
+      v[r] = k0 + r < nj ? ldi(pj + k0 + r) : -1;
+      du[r] = k0 + r < ni ? __ldcg(di + k0 + r) : (T)0;
+      dv[r] = k0 + r < nj ? __ldcg(dj + k0 + r) : (T)0;
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      su[r] = u[r] >= 0 ? __ldg(a.S + (size_t)u[r] * a.ld + j) : (T)0;
+      sv[r] = v[r] >= 0 ? __ldg(a.S + (size_t)v[r] * a.ld + i) : (T)0;
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (u[r] >= 0) wij = fma_t(du[r], su[r], wij);
+      if (v[r] >= 0) wji = fma_t(dv[r], sv[r], wji);
+    }
+  }
 }
 
 // Brings every stored row with pending entries up to date, in place: two work
@@ -550,22 +606,51 @@ __device__ __noinline__ void verify_pass(const ScreenArgs<T>& a, const T* __rest
   }
 }
 
-}  // namespace
+// ---- the group of CTAs that runs a launch: the whole cooperative grid, or
+// one thread-block cluster.  A grid barrier is an atomic and a polled word in
+// L2 (~1.5 us with 152 CTAs), a cluster barrier a hardware one (~0.3 us); a
+// sweep of a small problem is a chain of some twenty of them.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
 
-template <typename T, bool MIXED>
-__global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs<T> a) {
+// As round_barrier_any over a cluster of G <= kMaxCluster CTAs: every CTA's
+// flag into every CTA's shared memory, one barrier.  `par` alternates, so a
+// round's flags are read while the next round's are written elsewhere.
+__device__ __forceinline__ bool cluster_any(bool flag, int G, int cta, int par) {
+  __shared__ int s_flags[2][kMaxCluster];
+  const int f = __syncthreads_or(flag) != 0 ? 1 : 0;
+  if ((int)threadIdx.x < G) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(&s_flags[par][cta]);
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
+        "st.shared::cluster.u32 [r], %2;\n\t}" ::"r"(at),
+        "r"((unsigned)threadIdx.x), "r"(f)
+        : "memory");
+  }
+  cluster_barrier();
+  int any = 0;
+  for (int c = 0; c < G; ++c) any |= s_flags[par][c];
+  return any != 0;
+}
+
+// The sweeps of one problem by a group of G CTAs, this one the cta-th.
+template <typename T, bool MIXED, bool CL>
+__device__ __forceinline__ void screened_body(const ScreenArgs<T>& a, const int G, const int cta) {
   using VT = Vec<T>;
   using VV = typename VT::V;
   constexpr int VN = VT::N;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gthreads = gridDim.x * blockDim.x;
-  const int gwarp = blockIdx.x * nwarps + wid, gwarps = gridDim.x * nwarps;
+  const int gtid = cta * blockDim.x + threadIdx.x, gthreads = G * blockDim.x;
+  const int gwarp = cta * nwarps + wid, gwarps = G * nwarps;
   // per-candidate loops take threads (warps) in this order: consecutive
   // candidates land on different CTAs, so a few thousand candidates spread
   // their scattered loads over every SM's load pipeline
-  const int sid = threadIdx.x * (int)gridDim.x + (int)blockIdx.x;
-  const int swarp = wid * (int)gridDim.x + (int)blockIdx.x;
+  const int sid = threadIdx.x * G + cta;
+  const int swarp = wid * G + cta;
   const int p = a.p, P = a.P, ld = a.ld;
   const ScreenWork<T>& w = a.w;
   const WaitCtl& wc = a.wait;
@@ -579,6 +664,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
   __shared__ double red[kScreenThreads / 32][kParts];
   __shared__ int s_tmp[32];
   __shared__ double s_res[kRes];
+  __shared__ double s_part[kParts];
   __shared__ int s_stop;
   __shared__ unsigned long long s_dmax;  // the CTA's largest rowacc + D_i of the sweep (bits)
   __shared__ unsigned long long s_qmax;  // the same over the rows that stay quiet (bits)
@@ -591,7 +677,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
   // the data checks of the kernels before this launch were not read by the
   // host yet: when one failed, end at once (every CTA reads the same word)
   if (a.input_flag != nullptr && ld_relaxed_s32(a.input_flag) != 0) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (cta == 0 && threadIdx.x == 0) {
       for (int k = 0; k < kRes; ++k) a.result[k] = 0.0;
       a.result[kResStatus] = 2.0;
       a.result[kResList] = -1.0;
@@ -600,12 +686,18 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
   }
   unsigned gen = 0;
   int where = 0;
+  auto group_sync = [&]() {
+    if constexpr (CL)
+      cluster_barrier();
+    else
+      grid_barrier(a.barrier, gen, wc, ++where);
+  };
   T* Wa = a.W;
   T* Wn = a.Wb;
   int cur = 0;
   int t = 0, first_delta = 0, since_best = 0;
   double best_kkt = 1e300;
-  int status = -1;  // set when the launch ends early (overflow: kStatusDense)
+  int status = -1;  // set when the launch ends early (kStatusDense)
   const bool kkt0 = a.kkt_only || a.n_sweeps <= 0;  // objective / KKT only
   int redo_total = 0;
   bool need_scan = true;  // row offsets of the current list still to be computed
@@ -639,8 +731,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
     for (int k = 0; k < kParts; ++k) v[k] = 0.0;
     screen_pass<T, MIXED>(a, Wa, cur, kkt0, lamd, v, lane, gwarp, gwarps);
     for (int i = gtid; i < p; i += gthreads) w.rowacc[i] = 0.0;
-    if (kkt0) reduce_parts(v, a.partials, red);
-    grid_barrier(a.barrier, gen, wc, ++where);
+    if (kkt0) reduce_parts(v, a.partials, red, cta);
+    group_sync();
   }
 
   for (;;) {
@@ -672,11 +764,11 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         //      when it reused its list: only the records are refreshed)
         if (!reuse) {
         if (need_scan) {  // else the previous sweep's reduce phase scanned the counts
-          if (blockIdx.x == 0) {
+          if (cta == 0) {
             cta_scan([&](int k) { return ldi(w.cnt_r[cur] + k); }, p, w.off_r, w.cur_r, s_tmp,
                      w.ctr + kCtrTermsPred);
           }
-          grid_barrier(a.barrier, gen, wc, ++where);
+          group_sync();
         }
         need_scan = true;
         if (ldi(w.ctr + kCtrTermsPred) > w.term_cap) {  // the terms cannot fit
@@ -689,7 +781,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
           w.row_ent[atomicAdd(w.cur_r + pr.x, 1)] = k;
           w.row_ent[atomicAdd(w.cur_r + pr.y, 1)] = k;
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         // each row's candidates in colour-step order, one warp per row: the
         // steps of a row are distinct (a colour step pairs the row with one
         // partner), so a candidate's position is the number of smaller steps;
@@ -743,7 +835,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
             }
           }
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         } else {
           need_scan = true;
         }
@@ -763,8 +855,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
             T* rec = w.nd_rec + 4 * (size_t)k;
             T w1 = __ldcg(Wa + (size_t)i * ld + j), w2 = __ldcg(Wa + (size_t)j * ld + i);
             if (have_pend) {  // the rows' deferred updates, in order
-              w1 = pend_fold(a, i, ldi(w.pend_n + i), j, w1);
-              w2 = pend_fold(a, j, ldi(w.pend_n + j), i, w2);
+              pend_fold2(a, i, j, ldi(w.pend_n + i), ldi(w.pend_n + j), w1, w2);
             }
             rec[0] = w1;
             rec[1] = w2;
@@ -785,23 +876,36 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
           int base = 0;
           if (lane == 31 && incl > 0) base = atomicAdd(w.ctr + kCtrTerms, incl);
           base = __shfl_sync(FULL, base, 31);
-          int tp = base + incl - cnt;
+          const int tp = base + incl - cnt;
           if (!valid) continue;
           w.term_ptr[k] = tp;
           if (tp + cnt > w.term_cap) continue;  // overflow: the sweep goes dense
-          for (int m = 0; m < pi; ++m, ++tp) {
-            const int q = ldi(w.row_ent + bi + m);
-            const int2 qp = __ldcg(cand + q);
-            const int u = qp.x == i ? qp.y : qp.x;
-            w.term_pred[tp] = q;
-            w.term_s[tp] = __ldg(a.S + (size_t)u * ld + j);
-          }
-          for (int m = 0; m < pj; ++m, ++tp) {
-            const int q = ldi(w.row_ent + bj + m);
-            const int2 qp = __ldcg(cand + q);
-            const int u = qp.x == j ? qp.y : qp.x;
-            w.term_pred[tp] = q;
-            w.term_s[tp] = __ldg(a.S + (size_t)u * ld + i);
+          // eight terms at a time: entry, pair and S entry are three loads
+          // that wait for one another, taken term by term ~1 us each
+          for (int m0 = 0; m0 < cnt; m0 += 8) {
+            int q[8];
+            T sv[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              const int m = m0 + x;
+              q[x] = m < cnt ? ldi(w.row_ent + (m < pi ? bi + m : bj + m - pi)) : -1;
+            }
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              const int r = m0 + x < pi ? i : j, c = m0 + x < pi ? j : i;
+              sv[x] = (T)0;
+              if (q[x] >= 0) {
+                const int2 qp = __ldcg(cand + q[x]);
+                const int u = qp.x == r ? qp.y : qp.x;
+                sv[x] = __ldg(a.S + (size_t)u * ld + c);
+              }
+            }
+#pragma unroll
+            for (int x = 0; x < 8; ++x)
+              if (q[x] >= 0) {
+                w.term_pred[tp + m0 + x] = q[x];
+                w.term_s[tp + m0 + x] = sv[x];
+              }
           }
         }
         if (gtid < kJacMax) w.jac[gtid] = 0;
@@ -809,7 +913,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         if (gtid == 0) {
           w.ctr[kCtrJacDone] = 0;
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         if (ldi(w.ctr + kCtrTerms) > w.term_cap) {
           status = kStatusDense;
           break;
@@ -817,126 +921,187 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         // ---- chain, in parallel: the changes d solve d_k = F_k(d of the
         //      earlier candidates sharing row i or j), a system over a DAG in
         //      colour-step order whose unique solution is the sequential
-        //      walk's.  Iterating d <- F(d) from d = 0 over all candidates at
-        //      once reaches it exactly: once an iteration leaves every d
-        //      unchanged (bit for bit) the iterate satisfies the system.  Each
-        //      link scales a perturbation by |s_uj| / (s_ii + s_jj), so the
-        //      iteration settles after a few dozen rounds instead of one
-        //      round per link.  Thread gtid owns candidate gtid (operands in
-        //      registers); further candidates (N > threads) reload theirs.
+        //      walk's.  Every candidate is evaluated again and again, in
+        //      place, from whatever values its predecessors have by then.
+        //      Once no d changed between two barriers (bit for bit), every
+        //      evaluation of that interval saw the final values, so they
+        //      satisfy the system: the result does not depend on the order.
+        //      Each link scales a perturbation by |s_uj| / (s_ii + s_jj), so
+        //      this settles after a few dozen evaluations instead of one per
+        //      link.  A round costs a load and a store through L2, the FMA
+        //      chain and the barrier: 1.9 us at p = 1000, 1.7 at p = 5000
+        //      (FP32).  Term by term from L2 (three loads that wait for one
+        //      another) it was 10 and 4.4 us; several evaluations between two
+        //      barriers took longer than they saved.  Candidates beyond the
+        //      owned ones (N > threads) reload their operands.
         // only the CTAs that own candidates iterate (barrier among them);
-        // the others wait at the phase's closing grid barrier.  Only the
-        // first kJacThreads threads of a CTA own candidates (enough for one
-        // candidate per thread over all SMs, at least two warps), so that
+        // the others wait at the phase's closing grid barrier.  A CTA owns
+        // just enough candidates that all SMs together own them all, so that
         // the rounds' scattered loads (and in FP64 the division of Eq. 3,
         // FP64 throughput per SM being small on this part) spread over the
         // SMs
-        const int kJacThreads =
-            min(kScreenThreads, max(64, ((N + (int)gridDim.x - 1) / (int)gridDim.x + 31) / 32 * 32));
-        const int jac_ctas = min((int)gridDim.x, (N + kJacThreads - 1) / kJacThreads);
-        const int jac_span = jac_ctas * kJacThreads;  // candidates owned one per thread
-        if ((int)blockIdx.x < jac_ctas) {
-          const int k0 = (int)threadIdx.x < kJacThreads ? (int)blockIdx.x * kJacThreads + (int)threadIdx.x
-                                                      : N;
+        const int own_n = min(kScreenThreads, max(32, ((N + G - 1) / G + 31) / 32 * 32));
+        // (every CTA of a cluster: its barrier takes them all)
+        const int jac_ctas = CL ? G : min(G, (N + own_n - 1) / own_n);
+        const int jac_span = jac_ctas * own_n;  // candidates owned
+        if (cta < jac_ctas) {
+          // thread c owns candidate c of the CTA's; `lanes` neighbouring
+          // threads (fewer candidates: more of them, 1 .. 16) request its
+          // predecessors' changes together and leave the nonzero ones, few
+          // near a solution, in order in shared memory.  (Applying them on
+          // one lane of each group would issue every FP64 operation for 2 of
+          // 32 lanes.)
+          int lanes = 1;
+          while (lanes < 16 && own_n * lanes * 2 <= kScreenThreads) lanes *= 2;
+          const int c = (int)threadIdx.x / lanes, l = (int)threadIdx.x % lanes;
+          // term x of candidate c, at c stride + x: its S entry and its
+          // candidate; the packed terms' changes and x; the rest in L2
+          const int stride =
+              ((int)(screened_dyn_smem(MIXED) / (own_n * (2 * sizeof(T) + 6))) - 2) | 1;
+          T* const sm_s = reinterpret_cast<T*>(dyn);
+          T* const sm_d = sm_s + own_n * stride;
+          int* const sm_q = reinterpret_cast<int*>(sm_d + own_n * stride);
+          unsigned short* const sm_x = reinterpret_cast<unsigned short*>(sm_q + own_n * stride);
+          unsigned short* const sm_n = sm_x + own_n * stride;  // 2 c: packed terms; + 1: of row i
+          const int glane = lane & ~(lanes - 1);  // the group's first lane
+          const unsigned below = ((1u << lane) - 1u) & ~((1u << glane) - 1u);
+          const unsigned group = ((1u << lanes) - 1u) << glane;
+          int ns = 0, ts = 0;  // terms of candidate c in shared memory; terms of its row i
+          if (c < own_n && cta * own_n + c < N) {
+            const int k = cta * own_n + c, t0 = ldi(w.term_ptr + k);
+            ts = ldi(w.nd_pi + k);
+            ns = min(ts + ldi(w.nd_pj + k), stride);
+#pragma unroll 4
+            for (int x = l; x < ns; x += lanes) {
+              sm_q[c * stride + x] = ldi(w.term_pred + t0 + x);
+              sm_s[c * stride + x] = __ldcg(w.term_s + t0 + x);
+            }
+          }
+          const int ns_warp = __reduce_max_sync(FULL, ns);
+          // the owned candidate
+          const int k0 = (int)threadIdx.x < own_n ? cta * own_n + (int)threadIdx.x : N;
           const bool own = k0 < N;
           T w1 = (T)0, w2 = (T)0, om = (T)0, ss = (T)1;
-          int t0 = 0, ts = 0, nt = 0;
-          int tpr[4] = {0, 0, 0, 0};
-          T tsv[4] = {(T)0, (T)0, (T)0, (T)0};
+          int tx = 0, nx = 0, sx = 0;  // its terms in L2: first, how many, of row i
           if (own) {
             const T* rec = w.nd_rec + 4 * (size_t)k0;
             w1 = __ldcg(rec);
             w2 = __ldcg(rec + 1);
             om = __ldcg(rec + 2);
             ss = __ldcg(rec + 3);
-            t0 = ldi(w.term_ptr + k0);
             const int pi = ldi(w.nd_pi + k0);
-            ts = t0 + pi;
-            nt = pi + ldi(w.nd_pj + k0);
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-              if (x < nt) {
-                tpr[x] = ldi(w.term_pred + t0 + x);
-                tsv[x] = __ldcg(w.term_s + t0 + x);
-              }
+            nx = pi + ldi(w.nd_pj + k0) - stride;
+            sx = pi - stride;
+            tx = ldi(w.term_ptr + k0) + stride;
           }
-          T dmine = (T)0;
-          const T* dcur = w.nd_delta;
-          T* dnext = w.nd_d2;
+          // W_ij and W_ji after n terms from L2: eight predecessors' changes
+          // are requested at a time and applied in order
+          auto fold = [&](int tp, int n, int split, T& vij, T& vji) {
+            for (int x0 = 0; x0 < n; x0 += 8) {
+              T d[8], sv[8];
+#pragma unroll
+              for (int x = 0; x < 8; ++x) {
+                d[x] = x0 + x < n ? ld_relaxed(w.nd_delta + ldi(w.term_pred + tp + x0 + x)) : (T)0;
+                sv[x] = x0 + x < n ? __ldcg(w.term_s + tp + x0 + x) : (T)0;
+              }
+#pragma unroll
+              for (int x = 0; x < 8; ++x)
+                if (d[x] != (T)0) {
+                  if (x0 + x < split)
+                    vij = fma_t(d[x], sv[x], vij);
+                  else
+                    vji = fma_t(d[x], sv[x], vji);
+                }
+            }
+          };
+          T dmine = (T)0, vi0 = nan_t((T)0), vj0 = nan_t((T)0);
           for (int r = 0; r < kJacMax; ++r) {
             bool changed = false;
+            {
+              int cnt = 0, split = 0;
+              for (int x0 = 0; x0 < ns_warp; x0 += 4 * lanes) {
+                T d[4];
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                  const int x = x0 + y * lanes + l;
+                  d[y] = x < ns ? ld_relaxed(w.nd_delta + sm_q[c * stride + x]) : (T)0;
+                }
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                  const int x = x0 + y * lanes + l;
+                  const unsigned m = __ballot_sync(FULL, d[y] != (T)0) & group;
+                  const unsigned mi = __ballot_sync(FULL, d[y] != (T)0 && x < ts) & group;
+                  if (d[y] != (T)0) {
+                    const int at = c * stride + cnt + __popc(m & below);
+                    sm_d[at] = d[y];
+                    sm_x[at] = (unsigned short)x;
+                  }
+                  cnt += __popc(m);
+                  split += __popc(mi);
+                }
+              }
+              if (l == 0 && c < own_n) {
+                sm_n[2 * c] = (unsigned short)cnt;
+                sm_n[2 * c + 1] = (unsigned short)split;
+              }
+            }
+            __syncthreads();
             if (own) {
               T vij = w1, vji = w2;
-#pragma unroll
-              for (int x = 0; x < 4; ++x)
-                if (x < nt) {
-                  const T d = __ldcg(dcur + tpr[x]);
-                  if (d != (T)0) {
-                    if (t0 + x < ts)
-                      vij = fma_t(d, tsv[x], vij);
-                    else
-                      vji = fma_t(d, tsv[x], vji);
-                  }
-                }
-              for (int x = 4; x < nt; ++x) {
-                const T d = __ldcg(dcur + ldi(w.term_pred + t0 + x));
-                if (d != (T)0) {
-                  if (t0 + x < ts)
-                    vij = fma_t(d, __ldcg(w.term_s + t0 + x), vij);
-                  else
-                    vji = fma_t(d, __ldcg(w.term_s + t0 + x), vji);
-                }
-              }
-              const T xv = (ss * om - vij) - vji;
-              const T sx = soft(xv, lam);
-              T nw = (T)0;
-              if (sx != (T)0) nw = sx / ss;
-              const T delta = nw - om;
-              changed = !same_bits(delta, dmine);
-              dmine = delta;
-              dnext[k0] = delta;
-              w.nd_new[k0] = nw;
-            }
-            for (int k = k0 + jac_span; k < N; k += jac_span) {
-              const T* rec = w.nd_rec + 4 * (size_t)k;
-              const int u0 = ldi(w.term_ptr + k), us = u0 + ldi(w.nd_pi + k),
-                        u1 = us + ldi(w.nd_pj + k);
-              T vij = __ldcg(rec), vji = __ldcg(rec + 1);
-              const T omk = __ldcg(rec + 2), ssk = __ldcg(rec + 3);
-              for (int x = u0; x < u1; ++x) {
-                const T d = __ldcg(dcur + ldi(w.term_pred + x));
-                if (d != (T)0) {
-                  if (x < us)
-                    vij = fma_t(d, __ldcg(w.term_s + x), vij);
-                  else
-                    vji = fma_t(d, __ldcg(w.term_s + x), vji);
+              const int at = (int)threadIdx.x * stride;
+              const int cnt = sm_n[2 * threadIdx.x], split = sm_n[2 * threadIdx.x + 1];
+#pragma unroll 4
+              for (int x = at; x < at + split; ++x) vij = fma_t(sm_d[x], sm_s[at + sm_x[x]], vij);
+#pragma unroll 4
+              for (int x = at + split; x < at + cnt; ++x) vji = fma_t(sm_d[x], sm_s[at + sm_x[x]], vji);
+              if (nx > 0) fold(tx, nx, sx, vij, vji);
+              // the same W entries give the same change (no division then)
+              if (!same_bits(vij, vi0) || !same_bits(vji, vj0)) {
+                vi0 = vij;
+                vj0 = vji;
+                const T xv = (ss * om - vij) - vji;
+                const T st = soft(xv, lam);
+                T nw = (T)0;
+                if (st != (T)0) nw = st / ss;
+                const T delta = nw - om;
+                w.nd_new[k0] = nw;
+                if (!same_bits(delta, dmine)) {
+                  dmine = delta;
+                  st_relaxed(w.nd_delta + k0, delta);
+                  changed = true;
                 }
               }
-              const T xv = (ssk * omk - vij) - vji;
-              const T sx = soft(xv, lam);
-              T nw = (T)0;
-              if (sx != (T)0) nw = sx / ssk;
-              const T delta = nw - omk;
-              changed |= !same_bits(delta, __ldcg(dcur + k));
-              dnext[k] = delta;
-              w.nd_new[k] = nw;
+              for (int k = k0 + jac_span; k < N; k += jac_span) {
+                const T* rec = w.nd_rec + 4 * (size_t)k;
+                const int u0 = ldi(w.term_ptr + k), pi = ldi(w.nd_pi + k), n = pi + ldi(w.nd_pj + k);
+                vij = __ldcg(rec);
+                vji = __ldcg(rec + 1);
+                const T omk = __ldcg(rec + 2), ssk = __ldcg(rec + 3);
+                fold(u0, n, pi, vij, vji);
+                const T xv = (ssk * omk - vij) - vji;
+                const T st = soft(xv, lam);
+                T nw = (T)0;
+                if (st != (T)0) nw = st / ssk;
+                const T delta = nw - omk;
+                w.nd_new[k] = nw;
+                if (!same_bits(delta, ld_relaxed(w.nd_delta + k))) {
+                  st_relaxed(w.nd_delta + k, delta);
+                  changed = true;
+                }
+              }
             }
-            const bool moved = round_barrier_any(w.jac + r, (unsigned)jac_ctas, changed, wc,
-                                                 ++where, (int)blockIdx.x);
-            const T* tmp = dcur;
-            dcur = dnext;
-            dnext = const_cast<T*>(tmp);
+            bool moved;
+            if constexpr (CL)
+              moved = cluster_any(changed, G, cta, r & 1);
+            else
+              moved = round_barrier_any(w.jac + r, (unsigned)jac_ctas, changed, wc, ++where, cta);
             if (!moved) {
-              // the solution sits in dcur; keep it in nd_delta
-              if (dcur != w.nd_delta)
-                for (int k = gtid; k < N; k += jac_ctas * (int)blockDim.x)
-                  w.nd_delta[k] = __ldcg(dcur + k);
               if (gtid == 0) w.ctr[kCtrJacDone] = 1;
               break;
             }
           }
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         if (ldi(w.ctr + kCtrJacDone) == 0) {
           // not settled: nothing changed yet, the dense kernel takes the sweep
           status = kStatusDense;
@@ -957,7 +1122,9 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         // (one thread per row, rows spread over the CTAs: the row's loads are
         // a few dependent levels, so all rows proceed at once; the FMAs run
         // in the same order as the dense kernel's)
-        for (int i = threadIdx.x * (int)gridDim.x + (int)blockIdx.x; i < p; i += gthreads) {
+        unsigned long long qmax = 0ull, dmaxb = 0ull;
+        int fill = 0;
+        for (int i = threadIdx.x * G + cta; i < p; i += gthreads) {
           const int b = ldi(w.off_r + i), ne = ldi(w.off_r + i + 1) - b;
           const int np = have_pend ? ldi(w.pend_n + i) : 0;
           int* pu = w.pend_u + (size_t)i * kPendRow;
@@ -1032,9 +1199,9 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
               const int slot = atomicAdd(w.ctr + kCtrLoud, 1);
               if (slot < kLoudMax) w.loud[slot] = i;
             } else {
-              atomicMax(&s_qmax, (unsigned long long)__double_as_longlong(ai));
+              qmax = max(qmax, (unsigned long long)__double_as_longlong(ai));
             }
-            if (rows_valid) atomicMax(&s_dmax, (unsigned long long)__double_as_longlong(ai));
+            if (rows_valid) dmaxb = max(dmaxb, (unsigned long long)__double_as_longlong(ai));
             int need = np + nchg;
             if (dd != (T)0) {
               if (need < kPendRow) {
@@ -1044,14 +1211,26 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
               ++need;
             }
             w.pend_new[i] = need;
-            atomicMax(&s_fill, need);
+            fill = max(fill, need);
           }
+        }
+        // (one shared-memory maximum per warp: per row, they queued up)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          qmax = max(qmax, __shfl_xor_sync(FULL, qmax, o));
+          dmaxb = max(dmaxb, __shfl_xor_sync(FULL, dmaxb, o));
+          fill = max(fill, __shfl_xor_sync(FULL, fill, o));
+        }
+        if (lane == 0 && (qmax | dmaxb | (unsigned)fill) != 0ull) {
+          atomicMax(&s_qmax, qmax);
+          atomicMax(&s_dmax, dmaxb);
+          atomicMax(&s_fill, fill);
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-          w.dpart[blockIdx.x] = __longlong_as_double((long long)s_dmax);
-          w.apart[blockIdx.x] = __longlong_as_double((long long)s_qmax);
-          w.dfill[blockIdx.x] = s_fill;
+          w.dpart[cta] = __longlong_as_double((long long)s_dmax);
+          w.apart[cta] = __longlong_as_double((long long)s_qmax);
+          w.dfill[cta] = s_fill;
         }
         // ---- commit the candidates' new values (both triangles)
         for (int k = sid; k < N; k += gthreads) {
@@ -1065,7 +1244,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
             v[kPartActive] += 2.0;  // counted per owner, as the dense pass does
           }
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         // ---- lazy verification: every CTA forms the same decision.  A pair
         //      outside the list has moved by at most rowacc_i + rowacc_j (+
         //      this sweep's D_i + D_j) since it was screened.  LAZY (every
@@ -1077,23 +1256,35 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         //      as DEFER, and the pairs of those rows are verified and
         //      screened (partial_verify).  FULL: row pass with V,
         //      verification, fresh screen
-        if (threadIdx.x == 0) {
-          double dm = 0.0, qm = 0.0;
+        if (wid == 0) {
+          // the CTAs' maxima over warp 0's lanes, as integers (nonnegative
+          // values order by their bits): one thread's FP64 maxima over 152
+          // CTAs were ~6 us of every sweep
+          long long dmb = 0, qmb = 0;
           int fm = 0;
-          for (int c = 0; c < (int)gridDim.x; ++c) {
-            dm = fmax(dm, __ldcg(w.dpart + c));
-            qm = fmax(qm, __ldcg(w.apart + c));
+          for (int c = lane; c < G; c += 32) {
+            dmb = max(dmb, __double_as_longlong(__ldcg(w.dpart + c)));
+            qmb = max(qmb, __double_as_longlong(__ldcg(w.apart + c)));
             fm = max(fm, ldi(w.dfill + c));
           }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            dmb = max(dmb, __shfl_xor_sync(FULL, dmb, o));
+            qmb = max(qmb, __shfl_xor_sync(FULL, qmb, o));
+            fm = max(fm, __shfl_xor_sync(FULL, fm, o));
+          }
+          const double dm = __longlong_as_double(dmb), qm = __longlong_as_double(qmb);
           const int nl = ldi(w.ctr + kCtrLoud);
           const bool may = a.lazy_verify && rows_valid && !force_full;
           const bool all_quiet = may && nl == 0;
           const bool partial = may && nl > 0 && nl <= kLoudMax && fm <= kPendRow;
-          s_fast = all_quiet ? (fm <= kPendRow ? kModeDefer : kModeLazy)
-                             : (partial ? kModePartial : kModeFull);
-          // largest rowacc after the sweep (verified rows restart from 0)
-          s_dsweep = partial ? qm : dm;
-          s_nloud = nl;
+          if (lane == 0) {
+            s_fast = all_quiet ? (fm <= kPendRow ? kModeDefer : kModeLazy)
+                               : (partial ? kModePartial : kModeFull);
+            // largest rowacc after the sweep (verified rows restart from 0)
+            s_dsweep = partial ? qm : dm;
+            s_nloud = nl;
+          }
         }
         __syncthreads();
         mode = s_fast;
@@ -1108,7 +1299,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         } else {
           if (have_pend) {  // the stored rows catch up before the row pass reads them
             flush_pending(a, Wa, lane, gwarp, gwarps);
-            grid_barrier(a.barrier, gen, wc, ++where);
+            group_sync();
             for (int i = gtid; i < p; i += gthreads) w.pend_n[i] = 0;
             have_pend = false;
           }
@@ -1280,7 +1471,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
               __syncwarp();
             }
           }
-          grid_barrier(a.barrier, gen, wc, ++where);
+          group_sync();
         }
         // ---- the new diagonal
         for (int k = gtid; k < p; k += gthreads) {
@@ -1309,8 +1500,9 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
             const T omk = d != (T)0 ? __ldcg(w.nd_new + k) : __ldcg(w.nd_rec + 4 * (size_t)k + 2);
             T w1, w2;
             if (deferred) {
-              w1 = pend_fold(a, i, ldi(w.pend_new + i), j, __ldcg(Wa + (size_t)i * ld + j));
-              w2 = pend_fold(a, j, ldi(w.pend_new + j), i, __ldcg(Wa + (size_t)j * ld + i));
+              w1 = __ldcg(Wa + (size_t)i * ld + j);
+              w2 = __ldcg(Wa + (size_t)j * ld + i);
+              pend_fold2(a, i, j, ldi(w.pend_new + i), ldi(w.pend_new + j), w1, w2);
             } else {
               w1 = __ldcg(Wn + (size_t)i * ld + j);
               w2 = __ldcg(Wn + (size_t)j * ld + i);
@@ -1325,7 +1517,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
           push_cand(next && !fast, i, j, w.cand[1 - cur], w.ctr + kCtrCand + 1 - cur,
                     w.cnt_r[1 - cur], w.nc_cap, lane);
         }
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         const int nf = ldi(w.ctr + kCtrFail);
         if (nf == 0) break;
         // ---- undo the sweep, add the failing pairs, redo
@@ -1356,17 +1548,17 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
         for (int k = 0; k < kParts; ++k) v[k] = 0.0;
         ++redo_total;
         reuse = false;  // the list grew: build it again
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         if (add < min(nf, w.fail_cap) || ++redo > a.max_redo) {
           status = kStatusDense;
           break;
         }
       }
-      if (status == kStatusDense) {
+      if (status >= 0) {
         // nothing of this sweep was kept; report the state as it stands
         break;
       }
-      reduce_parts(v, a.partials, red);
+      reduce_parts(v, a.partials, red, cta);
       // the per-row bounds after the sweep: 0 after a full verification,
       // and for the rows a partial one verified; else grown by D_i
       for (int i = gtid; i < p; i += gthreads)
@@ -1396,11 +1588,11 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
       if (mode == kModeFull) rows_valid = true;
       // row offsets of the next sweep's list (its pushes are complete); a
       // lazy sweep keeps its list, offsets and build
-      if (blockIdx.x == 0 && !fast) {
+      if (cta == 0 && !fast) {
         cta_scan([&](int k) { return ldi(w.cnt_r[1 - cur] + k); }, p, w.off_r, w.cur_r, s_tmp,
                  w.ctr + kCtrTermsPred);
       }
-      if (blockIdx.x == 0 && fast)  // fresh cursors for a later build of the kept list
+      if (cta == 0 && fast)  // fresh cursors for a later build of the kept list
         for (int k = threadIdx.x; k <= p; k += blockDim.x) w.cur_r[k] = ldi(w.off_r + k);
       need_scan = grew;  // a grown list is counted again by the next build
       acc = fast ? 2.0 * s_dsweep : 0.0;
@@ -1408,35 +1600,34 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
       n_lazy += fast ? 1 : 0;
       n_partial += mode == kModePartial ? 1 : 0;
       if (mode == kModeDefer || mode == kModePartial) have_pend = true;
-      grid_barrier(a.barrier, gen, wc, ++where);
+      group_sync();
     }
 
-    // ---------------- every CTA reduces the partials identically (warp 0:
-    //                  lanes stride over the CTAs, then a fixed shuffle tree)
-    double kkt = 0.0, quad = 0.0, pen = 0.0, lg = 0.0, dl = 0.0, ac = 0.0, bad = 0.0;
-    if (wid == 0) {
-      for (int b = lane; b < (int)gridDim.x; b += 32) {
-        const double* q = a.partials + (size_t)b * kParts;
-        kkt = fmax(kkt, __ldcg(q + kPartKkt));
-        quad += __ldcg(q + kPartQuad);
-        pen += __ldcg(q + kPartPen);
-        lg += __ldcg(q + kPartLog);
-        dl = fmax(dl, __ldcg(q + kPartDelta));
-        ac += __ldcg(q + kPartActive);
-        bad += __ldcg(q + kPartBad);
-      }
+    // ---------------- every CTA reduces the partials identically (one warp
+    //                  per part: lanes stride over the CTAs, then a fixed
+    //                  shuffle tree)
+    if (wid < kParts) {
+      const double* q = a.partials + wid;
+      if (wid == kPartKkt || wid == kPartDelta) {  // maxima of nonnegative values, by their bits
+        long long m = 0;
+        for (int b = lane; b < G; b += 32)
+          m = max(m, __double_as_longlong(__ldcg(q + (size_t)b * kParts)));
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        kkt = fmax(kkt, __shfl_xor_sync(FULL, kkt, o));
-        dl = fmax(dl, __shfl_xor_sync(FULL, dl, o));
-        quad += __shfl_xor_sync(FULL, quad, o);
-        pen += __shfl_xor_sync(FULL, pen, o);
-        lg += __shfl_xor_sync(FULL, lg, o);
-        ac += __shfl_xor_sync(FULL, ac, o);
-        bad += __shfl_xor_sync(FULL, bad, o);
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(FULL, m, o));
+        if (lane == 0) s_part[wid] = __longlong_as_double(m);
+      } else {
+        double x = 0.0;
+        for (int b = lane; b < G; b += 32) x += __ldcg(q + (size_t)b * kParts);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+        if (lane == 0) s_part[wid] = x;
       }
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
+      const double kkt = s_part[kPartKkt], quad = s_part[kPartQuad], pen = s_part[kPartPen],
+                   lg = s_part[kPartLog], dl = s_part[kPartDelta], ac = s_part[kPartActive],
+                   bad = s_part[kPartBad];
       const double obj = -lg + 0.5 * quad + lamd * pen;
       const bool aborted = ld_relaxed_s32(wc.abort) != 0;
       const bool nonfinite = bad > 0.0 || !isfinite(obj) || !isfinite(kkt);
@@ -1479,7 +1670,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
                 sweeps_done >= a.n_sweeps || dense_next)
                    ? 1
                    : 0;
-      if (blockIdx.x == 0) {
+      if (cta == 0) {
         if (do_sweep && tt < a.hist_len) {
           double* h = a.hist + (size_t)tt * kHist;
           h[0] = dl;
@@ -1540,11 +1731,11 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
       for (int k = gtid; k <= p; k += gthreads) w.cnt_r[cur][k] = 0;
       if (have_pend) {  // the screen reads the true W
         flush_pending(a, Wa, lane, gwarp, gwarps);
-        grid_barrier(a.barrier, gen, wc, ++where);
+        group_sync();
         for (int i = gtid; i < p; i += gthreads) w.pend_n[i] = 0;
         have_pend = false;
       }
-      grid_barrier(a.barrier, gen, wc, ++where);
+      group_sync();
       {
         double vz[kParts];
 #pragma unroll
@@ -1557,13 +1748,13 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
       need_scan = true;
       acc = 0.0;  // a fresh screen of the current iterate
       reuse = false;
-      grid_barrier(a.barrier, gen, wc, ++where);
+      group_sync();
       continue;
     }
     ++t;
   }
   // the last lambda's Omega (path)
-  if (a.path_n > 0 && status != kStatusDense && (int)s_res[kResStatus] != 2 &&
+  if (a.path_n > 0 && status < 0 && (int)s_res[kResStatus] != 2 &&
       (int)s_res[kResStatus] != 3 && !((int)s_res[kResStatus] == 4 && a.path_break_stall)) {
     if (a.path_om) {
       T* out = a.path_om + (size_t)pk * p * a.path_ldo;
@@ -1581,7 +1772,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
     }
   }
 
-  if (status == kStatusDense && blockIdx.x == 0 && threadIdx.x == 0) {
+  if (status >= 0 && cta == 0 && threadIdx.x == 0) {
     // the sweep in progress was undone or never started: t sweeps are done
     // (for a path: of lambda pk, whose index the host reads from kResPath)
     a.result[kResPath] = pk;
@@ -1593,13 +1784,13 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
     a.result[kResFirstDelta] = first_delta;
     a.result[kResRedo] = redo_total;
     a.result[kResList] = -1.0;
-    a.result[kResStatus] = ld_relaxed_s32(wc.abort) != 0 ? 3.0 : (double)kStatusDense;
+    a.result[kResStatus] = ld_relaxed_s32(wc.abort) != 0 ? 3.0 : (double)status;
   }
   // deferred updates into the stored rows, unless the host rebuilds W itself
   // (a dense hand-over always needs them)
-  if (have_pend && (a.keep_w || status == kStatusDense)) {
+  if (have_pend && (a.keep_w || status >= 0)) {
     flush_pending(a, Wa, lane, gwarp, gwarps);
-    grid_barrier(a.barrier, gen, wc, ++where);
+    group_sync();
   }
   // leave W in the caller's buffer
   if (Wa != a.W) {
@@ -1610,12 +1801,25 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs
   }
 }
 
-size_t screened_dyn_smem(bool mixed) {
-  // per warp: the row pass's staged changes (partner, step, delta), or (in
-  // another phase) the row sort's keys and steps
-  const size_t rows = (size_t)kRowList * (8 + (mixed ? 4 : 8));
-  const size_t sort = (size_t)2 * kSortCap * sizeof(int);
-  return (size_t)(kScreenThreads / 32) * (rows > sort ? rows : sort);
+}  // namespace
+
+template <typename T, bool MIXED>
+__global__ void __launch_bounds__(kScreenThreads, 1) k_screened(const ScreenArgs<T> a) {
+  screened_body<T, MIXED, false>(a, (int)gridDim.x, (int)blockIdx.x);
+}
+
+// One problem per cluster: problem blockIdx.x / cluster size of the table.
+// The clusters share nothing, so any number of them may wait for a place on
+// the device.
+template <typename T, bool MIXED>
+__global__ void __launch_bounds__(kScreenThreads, 1)
+    k_screened_batch(const ScreenArgs<T>* __restrict__ probs, const int size) {
+  __shared__ ScreenArgs<T> s_a;
+  const int* src = reinterpret_cast<const int*>(probs + blockIdx.x / size);
+  for (int e = threadIdx.x; e < (int)(sizeof(ScreenArgs<T>) / sizeof(int)); e += blockDim.x)
+    reinterpret_cast<int*>(&s_a)[e] = __ldg(src + e);
+  __syncthreads();
+  screened_body<T, MIXED, true>(s_a, size, (int)(blockIdx.x % size));
 }
 
 template <typename T, bool MIXED>
@@ -1634,6 +1838,74 @@ cudaError_t launch_screened(const ScreenArgs<double>& a, int grid, cudaStream_t 
 }
 cudaError_t launch_screened(const ScreenArgs<float>& a, int grid, cudaStream_t st) {
   return launch_screened_impl<float, true>(a, grid, st);
+}
+
+template <typename... A>
+cudaError_t launch_clusters(void (*fn)(A...), int grid, int size, size_t dyn, cudaStream_t st,
+                            A... args) {
+  cudaError_t e =
+      cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kScreenThreads);
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = size;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  note_launches(1);
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
+cudaError_t launch_screened_batch(const ScreenArgs<double>* probs, int n, int size, cudaStream_t st) {
+  return launch_clusters<const ScreenArgs<double>*, int>(k_screened_batch<double, false>, n * size,
+                                                         size, screened_dyn_smem(false), st, probs,
+                                                         size);
+}
+cudaError_t launch_screened_batch(const ScreenArgs<float>* probs, int n, int size, cudaStream_t st) {
+  return launch_clusters<const ScreenArgs<float>*, int>(k_screened_batch<float, true>, n * size, size,
+                                                        screened_dyn_smem(true), st, probs, size);
+}
+
+// Largest launchable cluster (a power of two <= kMaxCluster; 0 if none).
+cudaError_t screened_cluster_size(bool mixed, int* size) {
+  const size_t dyn = screened_dyn_smem(mixed);
+  const void* fn = mixed ? (const void*)k_screened_batch<float, true>
+                         : (const void*)k_screened_batch<double, false>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  *size = 0;
+  for (int c = kMaxCluster; c >= 2; c >>= 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(kScreenThreads);
+    cfg.dynamicSmemBytes = dyn;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    e = mixed ? cudaOccupancyMaxActiveClusters(&n, k_screened_batch<float, true>, &cfg)
+              : cudaOccupancyMaxActiveClusters(&n, k_screened_batch<double, false>, &cfg);
+    if (e == cudaSuccess && n >= 1) {
+      *size = c;
+      return cudaSuccess;
+    }
+    cudaGetLastError();
+  }
+  return cudaSuccess;
 }
 
 cudaError_t screened_occupancy(bool mixed, int* blocks_per_sm) {
