@@ -754,7 +754,8 @@ int concord_joint_get_history(concord_joint *jt, double *hist_host, int max_rows
  * A batch holds many independent CONCORD problems (dimensions p[b], uneven
  * allowed; data of uneven n) and solves them together: one persistent
  * cooperative launch of the sweep kernel per wave of problems whose CTAs fit
- * co-resident on the device, all problems of a wave in flight at once.  In
+ * co-resident on the device, all problems of a wave in flight at once (or,
+ * by default, one cluster per problem, see concord_batch_path).  In
  * the launch every problem owns a contiguous range of CTAs (its rows,
  * mailbox ring, barrier counter and partial sums are its own), runs
  * Algorithm 1's colour steps and diagonal step (Section 3.2, 3.3; Eq. 2,
@@ -819,19 +820,22 @@ int concord_batch_reset(concord_batch *bt, int b);
  * CONCORD_NOT_CONVERGED; MIXED: sweeps_fp32 = its FP32 sweeps).
  * support_dev (device, nullable; all problems of one
  * p) gains, for every problem and lambda k, 1.0 at [k][i][j] where
- * w_ij != 0 (n_lambda x p x p floats, not cleared by the call).  When the
- * rows per warp are not set, the call first autotunes them
- * (concord_batch_autotune at the middle lambda, which resets every problem
- * to Omega = I).  Synchronises the stream.
+ * w_ij != 0 (n_lambda x p x p floats, not cleared by the call).  Unless a
+ * layout was set (concord_batch_set_rows_per_warp), the sweeps are screened
+ * ones (CONCORD_SWEEP_SCREENED), one thread-block cluster per problem in one
+ * launch; a lambda whose candidate list is too long runs on the dense kernel
+ * and the walk resumes after it.  Same iterates either way.  Synchronises the
+ * stream.
  * Errors: CONCORD_E_ARG, CONCORD_E_OCCUPANCY, CONCORD_E_TIMEOUT, CONCORD_E_CUDA. */
 int concord_batch_path(concord_batch *bt, const double *lambdas, int n_lambda, double tol,
                        int max_sweeps, concord_result *results, float *support_dev);
 
-/* The batch's work layout: each warp of a problem owns up to `rows` rows
- * (2, 4, 8, 16 or 32; 0: autotune on the next concord_batch_path), so a
- * problem of dimension p takes ceil(p / (16 rows)) CTAs of 512 threads and
- * fewer rows per warp trade co-resident problems (waves) for row-update
- * bandwidth.  Results do not depend on it. */
+/* Every sweep on the dense kernel, in this work layout: each warp of a problem
+ * owns up to `rows` rows (2, 4, 8, 16 or 32), so a problem of dimension p
+ * takes ceil(p / (16 rows)) CTAs of 512 threads and fewer rows per warp trade
+ * co-resident problems (waves) for row-update bandwidth.  0 (the default):
+ * screened sweeps, and the next concord_batch_path starts from Omega = I
+ * again.  Results do not depend on it. */
 int concord_batch_set_rows_per_warp(concord_batch *bt, int rows);
 
 /* MIXED: FP64 polish of stalled lambdas in concord_batch_path (1, the
@@ -840,12 +844,13 @@ int concord_batch_set_polish(concord_batch *bt, int on);
 
 /* Times `sweeps` sweeps at `lambda` on every problem for each rows-per-warp
  * choice (32, 16, 8, 4, 2; ms_per_choice, host, nullable, receives the five
- * times in ms, -1 where a choice cannot launch), keeps the fastest, and
- * resets every problem to Omega = I.  Errors: as concord_batch_path. */
+ * times in ms, -1 where a choice cannot launch), keeps the fastest for the
+ * sweeps that run on the dense kernel, and resets every problem to Omega = I.
+ * Errors: as concord_batch_path. */
 int concord_batch_autotune(concord_batch *bt, double lambda, int sweeps, double *ms_per_choice);
 
-/* The layout of the last launch: rows per warp, the largest wave's CTAs,
- * the number of waves, and the device time of the last path (or trial). */
+/* The layout of the last launch: rows per warp of the dense kernel (0: not
+ * chosen), the largest wave's CTAs, the number of waves, and the device time of the last path (or trial). */
 int concord_batch_info(concord_batch *bt, int *rows_per_warp, int *ctas, int *waves,
                        double *seconds);
 

@@ -1,7 +1,9 @@
 // Host side of the batched entry points (concord_batch_*) of the C ABI in
-// include/concord.h: many independent CONCORD problems (uneven p and n) in
-// one persistent launch of the sweep kernel per wave of co-resident
-// problems, each problem walking a warm-started lambda path.
+// include/concord.h: many independent CONCORD problems (uneven p and n), each
+// walking a warm-started lambda path: screened sweeps with one thread-block
+// cluster per problem in one launch, and the lambdas whose candidate lists
+// are too long (or all, when the caller set a layout) on the dense sweep
+// kernel, one persistent launch per wave of co-resident problems.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
@@ -14,6 +16,7 @@
 #include "concord.h"
 #include "kernels.h"
 #include "prep_stats.h"
+#include "screen_scratch.h"
 
 using namespace concord;
 
@@ -44,6 +47,12 @@ int rup(int v, int m) { return (v + m - 1) / m * m; }
 
 constexpr int kBatchWarps = kSweepThreads / 32;  // warps per CTA, all owning rows
 constexpr int kRowsChoices[] = {32, 16, 8, 4, 2};
+constexpr int kDenseRows = 8;  // dense layout of a screened batch that was not autotuned
+// Candidate pairs and correction terms of a problem's screened sweeps; a
+// lambda that needs more runs on the dense kernel.  Smaller than a single
+// state's: a problem has a few SMs here, and its dense sweeps run beside the
+// other problems'.
+constexpr int kBatchCandPerRow = 24, kBatchCandMin = 16384, kBatchTermsPerCand = 32;
 
 // One problem's device arrays (T = float for CONCORD_MIXED, double for FP64).
 struct Prob {
@@ -55,6 +64,12 @@ struct Prob {
   double *S64 = nullptr, *W64 = nullptr, *Om64 = nullptr, *sd1_64 = nullptr, *sd2_64 = nullptr;
   unsigned long long* mbox = nullptr;
   unsigned* barrier = nullptr;
+  float* mrow = nullptr;  // [p] m[u] >= max_{x != u} |s_ux| (lazy verification bound)
+  // screened sweeps (allocated on first use): W after the sweep, W at each
+  // pair's visit, the lists, per-CTA partial sums and the launch's result
+  void *Wb = nullptr, *V = nullptr, *scr = nullptr;
+  double* sres = nullptr;
+  int nc = 0, tc = 0;
   bool have_S = false;
 };
 
@@ -70,13 +85,16 @@ struct concord_batch {
   cudaStream_t stream = nullptr, own_stream = nullptr;
   std::vector<Prob> probs;
   double timeout_s = 2.0;
-  int rows_per_warp = 0;  // 0: autotune on the first path call
+  int rows_per_warp = 0;  // dense layout; 0: not chosen
+  bool reset_next = false;  // the layout was given back: the next path starts from Omega = I
+  bool rows_set = false;  // chosen by the caller: every sweep runs on the dense kernel
   bool polish = true;     // MIXED: FP64 polish of a lambda whose FP32 sweeps stall
   int last_ctas = 0, last_waves = 0;
   // data staging for concord_batch_gram (one problem at a time)
   double *Xg = nullptr, *mean = nullptr, *inv = nullptr, *part = nullptr;
   float *zt_hi = nullptr, *zt_lo = nullptr;
   void* Z = nullptr;
+  void* gf_work = nullptr;  // FP64: digits and scales of the Gram
   int* flag = nullptr;
   int* h_flag = nullptr;
   // launch scratch
@@ -87,6 +105,7 @@ struct concord_batch {
   size_t res_cap = 0;
   void* probs_dev = nullptr;
   size_t probs_cap = 0;
+  int cluster_max = -1;  // largest launchable cluster (-1: not queried)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   float last_ms = 0.f;
 };
@@ -99,7 +118,7 @@ size_t esz(const concord_batch* bt) { return is_mixed(bt) ? 4 : 8; }
 void free_prob(Prob& q) {
   void* d[] = {q.S,        q.W,      q.Om,     q.sdiagT, q.sd1,    q.sd2,  q.sdiag64,
                q.omdiag64, q.partials, q.mbox, q.barrier, q.S64, q.W64, q.Om64,
-               q.sd1_64,   q.sd2_64};
+               q.sd1_64,   q.sd2_64, q.mrow, q.Wb, q.V, q.scr, q.sres};
   for (void* x : d)
     if (x) cudaFree(x);
   q = Prob();
@@ -107,7 +126,7 @@ void free_prob(Prob& q) {
 
 void free_all(concord_batch* bt) {
   for (auto& q : bt->probs) free_prob(q);
-  void* d[] = {bt->Xg, bt->mean, bt->inv, bt->part, bt->zt_hi, bt->zt_lo, bt->Z, bt->flag, bt->abort_info,
+  void* d[] = {bt->Xg, bt->mean, bt->inv, bt->part, bt->zt_hi, bt->zt_lo, bt->Z, bt->gf_work, bt->flag, bt->abort_info,
                bt->lam_dev, bt->res_dev, bt->probs_dev};
   for (void* x : d)
     if (x) cudaFree(x);
@@ -139,6 +158,7 @@ int reset_prob(concord_batch* bt, Prob& q) {
   }
   BCK(launch_subdiag(q.S, f32, q.ld, q.p, q.P, q.sd1, q.sd2, s));
   if (f32) BCK(launch_subdiag(q.S64, 0, q.ld, q.p, q.P, q.sd1_64, q.sd2_64, s));
+  BCK(launch_row_absmax(q.S, f32, q.ld, q.p, q.mrow, s));
   BCK(launch_set_identity(q.Om, f32, q.p, q.ld, s));
   BCK(cudaMemcpyAsync(q.W, q.S, esz(bt) * (size_t)q.p * q.ld, cudaMemcpyDeviceToDevice, s));
   BCK(cudaMemcpyAsync(bt->h_flag, bt->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -153,6 +173,38 @@ int reset_prob(concord_batch* bt, Prob& q) {
 int ctas_for(int p, int rows) {
   const int per_cta = kBatchWarps * rows;
   return (p + per_cta - 1) / per_cta;
+}
+
+// Device copies of the lambdas, the (cleared) result rows and room for a
+// problem table.
+int ensure_tables(concord_batch* bt, const double* lambdas_host, int n_lambda, size_t table_bytes) {
+  cudaStream_t s = bt->stream;
+  if (n_lambda > bt->lam_cap) {
+    if (bt->lam_dev) cudaFree(bt->lam_dev);
+    bt->lam_dev = nullptr;
+    bt->lam_cap = 0;
+    BCK(cudaMalloc(&bt->lam_dev, sizeof(double) * n_lambda));
+    bt->lam_cap = n_lambda;
+  }
+  BCK(cudaMemcpyAsync(bt->lam_dev, lambdas_host, sizeof(double) * n_lambda,
+                      cudaMemcpyHostToDevice, s));
+  const size_t nres = bt->probs.size() * (size_t)n_lambda * kRes;
+  if (nres > bt->res_cap) {
+    if (bt->res_dev) cudaFree(bt->res_dev);
+    bt->res_dev = nullptr;
+    bt->res_cap = 0;
+    BCK(cudaMalloc(&bt->res_dev, sizeof(double) * nres));
+    bt->res_cap = nres;
+  }
+  BCK(cudaMemsetAsync(bt->res_dev, 0, sizeof(double) * nres, s));
+  if (table_bytes > bt->probs_cap) {
+    if (bt->probs_dev) cudaFree(bt->probs_dev);
+    bt->probs_dev = nullptr;
+    bt->probs_cap = 0;
+    BCK(cudaMalloc(&bt->probs_dev, table_bytes));
+    bt->probs_cap = table_bytes;
+  }
+  return CONCORD_OK;
 }
 
 // One launch per wave of co-resident items.  T = float: the FP32 arrays of
@@ -176,28 +228,9 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
       return bfail(CONCORD_E_ARG, "p=%d needs more than %d CTAs at %d rows per warp",
                    bt->probs[it.b].p, capacity, rows);
   // device copies of the lambdas, the result rows and the problem table
-  if (n_lambda > bt->lam_cap) {
-    if (bt->lam_dev) cudaFree(bt->lam_dev);
-    bt->lam_dev = nullptr;
-    BCK(cudaMalloc(&bt->lam_dev, sizeof(double) * n_lambda));
-    bt->lam_cap = n_lambda;
-  }
-  BCK(cudaMemcpyAsync(bt->lam_dev, lambdas_host, sizeof(double) * n_lambda,
-                      cudaMemcpyHostToDevice, s));
   const size_t nres = (size_t)B * n_lambda * kRes;
-  if (nres > bt->res_cap) {
-    if (bt->res_dev) cudaFree(bt->res_dev);
-    bt->res_dev = nullptr;
-    BCK(cudaMalloc(&bt->res_dev, sizeof(double) * nres));
-    bt->res_cap = nres;
-  }
-  BCK(cudaMemsetAsync(bt->res_dev, 0, sizeof(double) * nres, s));
-  if ((size_t)nI * sizeof(BatchProblem<T>) > bt->probs_cap) {
-    if (bt->probs_dev) cudaFree(bt->probs_dev);
-    bt->probs_dev = nullptr;
-    BCK(cudaMalloc(&bt->probs_dev, (size_t)nI * sizeof(BatchProblem<T>)));
-    bt->probs_cap = (size_t)nI * sizeof(BatchProblem<T>);
-  }
+  int rc = ensure_tables(bt, lambdas_host, n_lambda, (size_t)nI * sizeof(BatchProblem<T>));
+  if (rc != CONCORD_OK) return rc;
   // greedy waves of consecutive items whose CTAs fit co-resident
   std::vector<std::pair<int, int>> waves;
   {
@@ -304,6 +337,108 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
   return CONCORD_OK;
 }
 
+// Scratch of a problem's screened sweeps (allocated on first use).
+int ensure_screen(concord_batch* bt, Prob& q) {
+  if (q.scr) return CONCORD_OK;
+  const long long pairs = (long long)q.p * (q.p - 1) / 2;
+  long long nc = std::max((long long)kBatchCandPerRow * q.p, (long long)kBatchCandMin);
+  nc = std::max(1ll, std::min(nc, pairs));
+  q.nc = (int)nc;
+  q.tc = (int)std::min(nc * kBatchTermsPerCand, 1ll << 25);
+  const size_t mat = esz(bt) * (size_t)q.p * q.ld;
+  BCK(cudaMalloc(&q.Wb, mat));
+  BCK(cudaMalloc(&q.V, mat));
+  BCK(cudaMalloc((void**)&q.sres, sizeof(double) * (kRes + kMaxCluster * kParts)));
+  BCK(cudaMemsetAsync(q.Wb, 0, mat, bt->stream));
+  BCK(cudaMemsetAsync(q.V, 0, mat, bt->stream));
+  BCK(cudaMalloc(&q.scr, screen_layout(q.p, q.P, q.nc, q.tc).total));
+  return CONCORD_OK;
+}
+
+// One launch, one cluster per item (its problem's path lambdas[k0 .. k0 +
+// nk)).  Result rows as run_waves; ends[i]: the kRes values an item's walk
+// ended with (status kStatusDense: lambda kResPath, after kResSweeps sweeps,
+// needs the dense kernel; 4 with stall_break: it stalled).
+template <typename T>
+int run_screened(concord_batch* bt, const std::vector<Item>& items, const double* lambdas_host,
+                 int n_lambda, double tol, int max_sweeps, int stall_stop, float* support_dev,
+                 std::vector<double>* res_host, std::vector<double>* ends) {
+  cudaStream_t s = bt->stream;
+  const int nI = (int)items.size();
+  if (bt->cluster_max < 0) BCK(screened_cluster_size(sizeof(T) == 4, &bt->cluster_max));
+  // the SMs shared out evenly, up to the largest cluster: 24 problems of p =
+  // 500 on 6 CTAs each; a row's share of a CTA below 32 rows gains nothing
+  int size = std::max(1, std::min(bt->sms / nI, rup(bt->pmax, 32) / 32));
+  size = std::min(size, bt->cluster_max > 0 ? bt->cluster_max : 1);
+  if (size > 8) size = size >= 16 ? 16 : 8;  // beyond 8, only 16 is a launchable size
+  int rc = ensure_tables(bt, lambdas_host, n_lambda, (size_t)nI * sizeof(ScreenArgs<T>));
+  if (rc != CONCORD_OK) return rc;
+  std::vector<ScreenArgs<T>> table(nI);
+  for (int i = 0; i < nI; ++i) {
+    const Item& it = items[i];
+    Prob& q = bt->probs[it.b];
+    if ((rc = ensure_screen(bt, q)) != CONCORD_OK) return rc;
+    ScreenArgs<T>& a = table[i];
+    memset((void*)&a, 0, sizeof a);
+    a.p = q.p;
+    a.P = q.P;
+    a.ld = q.ld;
+    a.W = (T*)q.W;
+    a.Wb = (T*)q.Wb;
+    a.V = (T*)q.V;
+    a.Om = (T*)q.Om;
+    a.S = (const T*)q.S;
+    a.sdiag = (const T*)q.sdiagT;
+    a.sdiag64 = q.sdiag64;
+    a.omdiag64 = sizeof(T) == 4 ? q.omdiag64 : nullptr;
+    a.w = screen_work_at<T>(q.scr, q.p, q.P, q.nc, q.tc);
+    a.wait.abort = bt->abort_info;
+    a.wait.info = bt->abort_info + 1;
+    a.wait.timeout_ns = (uint64_t)(bt->timeout_s * 1e9);
+    a.result = q.sres;
+    a.partials = q.sres + kRes;
+    a.lambda = lambdas_host[it.k0];
+    a.tol = tol;
+    a.delta_tol = 1e-5;
+    a.stop_rule = CONCORD_STOP_KKT;
+    a.n_sweeps = max_sweeps;
+    a.stall_stop = stall_stop;
+    a.max_redo = 8;
+    a.start_list = -1;
+    a.path_lambda = bt->lam_dev;
+    a.path_n = it.k0 + it.nk;
+    a.path_start = it.k0;
+    a.path_res = bt->res_dev + (size_t)it.b * n_lambda * kRes;
+    a.path_cnt = support_dev;
+    a.mrow = q.mrow;
+    a.lazy_verify = 1;
+    a.keep_w = 1;
+    a.path_break_stall = it.stall_break;
+  }
+  BCK(cudaMemcpyAsync(bt->probs_dev, table.data(), (size_t)nI * sizeof(ScreenArgs<T>),
+                      cudaMemcpyHostToDevice, s));
+  BCK(cudaMemsetAsync(bt->abort_info, 0, 3 * sizeof(int), s));
+  BCK(cudaEventRecord(bt->ev0, s));
+  BCK(launch_screened_batch((const ScreenArgs<T>*)bt->probs_dev, nI, size, s));
+  BCK(cudaEventRecord(bt->ev1, s));
+  const size_t nres = bt->probs.size() * (size_t)n_lambda * kRes;
+  res_host->assign(nres, 0.0);
+  ends->assign((size_t)nI * kRes, 0.0);
+  BCK(cudaMemcpyAsync(res_host->data(), bt->res_dev, sizeof(double) * nres,
+                      cudaMemcpyDeviceToHost, s));
+  for (int i = 0; i < nI; ++i)
+    BCK(cudaMemcpyAsync(ends->data() + (size_t)i * kRes, bt->probs[items[i].b].sres,
+                        sizeof(double) * kRes, cudaMemcpyDeviceToHost, s));
+  BCK(cudaStreamSynchronize(s));
+  BCK(cudaGetLastError());
+  float ms = 0.f;
+  BCK(cudaEventElapsedTime(&ms, bt->ev0, bt->ev1));
+  bt->last_ms = ms;
+  bt->last_ctas = std::max(bt->last_ctas, std::min(nI * size, bt->sms));
+  bt->last_waves = std::max(bt->last_waves, (nI * size + bt->sms - 1) / bt->sms);
+  return CONCORD_OK;
+}
+
 std::vector<Item> all_items(const concord_batch* bt, int n_lambda, int stall_break) {
   std::vector<Item> items;
   for (int b = 0; b < (int)bt->probs.size(); ++b) items.push_back({b, 0, n_lambda, stall_break, 0});
@@ -339,70 +474,122 @@ int demote(concord_batch* bt, Prob& q) {
   return CONCORD_OK;
 }
 
-// The MIXED path with polish: the FP32 launches walk every problem's path
-// until a lambda's sweeps stall (the problem's walk ends there); those
-// lambdas are polished in FP64 (one launch for all of them), their support
-// counted from the FP64 iterate, and the walks resume after them.
-int mixed_path(concord_batch* bt, int rows, const double* lambdas, int n_lambda, double tol,
-               int max_sweeps, float* support_dev, std::vector<double>* R,
-               std::vector<int>* sweeps32) {
+// What a path call records beside the result rows, per problem and lambda.
+struct PathLog {
+  std::vector<double> rows;              // kRes values each
+  std::vector<int> sweeps32, dense;      // FP32 sweeps; sweeps on the dense kernel
+};
+
+// Every problem's path.  Unless the caller chose a dense layout, a launch
+// walks each on the screened sweeps; a lambda whose candidates overflow runs
+// on the dense kernel (with the other problems' that did), and the walk
+// resumes after it.  MIXED with polish: a lambda whose FP32 sweeps stall ends
+// the walk too; those lambdas are polished in FP64 (one launch for all of
+// them), their support counted from the FP64 iterate.
+template <typename T>
+int walk(concord_batch* bt, const double* lambdas, int n_lambda, double tol, int max_sweeps,
+         float* support_dev, PathLog* log) {
   const int B = (int)bt->probs.size();
-  R->assign((size_t)B * n_lambda * kRes, 0.0);
-  sweeps32->assign((size_t)B * n_lambda, 0);
+  const bool mixed = sizeof(T) == 4;
+  const int brk = mixed && bt->polish ? 1 : 0, stall = mixed ? 1 : 0;
+  const int rows = bt->rows_per_warp > 0 ? bt->rows_per_warp : kDenseRows;
+  const size_t cells = (size_t)B * n_lambda;
+  log->rows.assign(cells * kRes, 0.0);
+  log->sweeps32.assign(cells, 0);
+  log->dense.assign(cells, 0);
   std::vector<int> next(B, 0);
-  std::vector<double> res;
+  std::vector<double> res, ends;
   bt->last_ctas = bt->last_waves = 0;
   float total_ms = 0.f;
   for (;;) {
     std::vector<Item> items;
     for (int b = 0; b < B; ++b)
-      if (next[b] < n_lambda) items.push_back({b, next[b], n_lambda - next[b], 1, 0});
+      if (next[b] < n_lambda) items.push_back({b, next[b], n_lambda - next[b], brk, 0});
     if (items.empty()) break;
-    int rc = run_waves<float>(bt, rows, items, lambdas, n_lambda, tol, max_sweeps, 1, support_dev,
-                              &res);
-    if (rc != CONCORD_OK) return rc;
-    total_ms += bt->last_ms;
-    std::vector<Item> pol;
-    for (const Item& it : items) {
-      int k = it.k0;
-      for (; k < n_lambda; ++k) {
-        const double* x = res.data() + ((size_t)it.b * n_lambda + k) * kRes;
-        const size_t o = ((size_t)it.b * n_lambda + k) * kRes;
-        for (int q = 0; q < kRes; ++q) (*R)[o + q] = x[q];
-        (*sweeps32)[(size_t)it.b * n_lambda + k] = (int)x[kResSweeps];
-        const int code = (int)x[kResStatus];
-        if (code == 4) break;              // stalled: polish it
-        if (code == 2 || code == 3) {      // non-finite / aborted: the walk ended
-          k = n_lambda;
-          break;
+    // a problem's rows up to (and with) the lambda its walk ended at
+    auto take = [&](const Item& it, int k, int before, bool dense) {
+      const size_t o = (size_t)it.b * n_lambda + k;
+      for (int q = 0; q < kRes; ++q) log->rows[o * kRes + q] = res[o * kRes + q];
+      log->rows[o * kRes + kResSweeps] += before;
+      if (mixed) log->sweeps32[o] = (int)log->rows[o * kRes + kResSweeps];
+      if (dense) log->dense[o] = (int)res[o * kRes + kResSweeps];
+      return (int)res[o * kRes + kResStatus];
+    };
+    std::vector<Item> pol, dense;
+    std::vector<int> before;  // screened sweeps already done at a dense item's lambda
+    int rc;
+    if (bt->rows_set) {
+      rc = run_waves<T>(bt, rows, items, lambdas, n_lambda, tol, max_sweeps, stall, support_dev, &res);
+      if (rc != CONCORD_OK) return rc;
+      total_ms += bt->last_ms;
+      for (const Item& it : items) {
+        next[it.b] = n_lambda;
+        for (int k = it.k0; k < n_lambda; ++k) {
+          const int code = take(it, k, 0, true);
+          if (code == 2 || code == 3) break;  // non-finite / aborted: the walk ended
+          if (code == 4 && brk) {
+            pol.push_back({it.b, k, 1, 0, 0});
+            break;
+          }
         }
       }
-      if (k < n_lambda) {
-        const int done = (*sweeps32)[(size_t)it.b * n_lambda + k];
-        pol.push_back({it.b, k, 1, 0, max_sweeps > done ? max_sweeps - done : 1});
-        next[it.b] = k;
-      } else {
+    } else {
+      rc = run_screened<T>(bt, items, lambdas, n_lambda, tol, max_sweeps, stall, support_dev, &res,
+                           &ends);
+      if (rc != CONCORD_OK) return rc;
+      total_ms += bt->last_ms;
+      for (size_t i = 0; i < items.size(); ++i) {
+        const Item& it = items[i];
+        const double* e = ends.data() + i * kRes;
+        const int code = (int)e[kResStatus], last = (int)e[kResPath];
         next[it.b] = n_lambda;
+        for (int k = it.k0; k < (code == kStatusDense ? last : last + 1); ++k) take(it, k, 0, false);
+        if (code == kStatusDense) {
+          const int done = (int)e[kResSweeps];
+          dense.push_back({it.b, last, 1, brk, max_sweeps > done ? max_sweeps - done : 1});
+          before.push_back(done);
+        } else if (code == 4 && brk) {
+          pol.push_back({it.b, last, 1, 0, 0});
+        }
+      }
+      if (!dense.empty()) {
+        rc = run_waves<T>(bt, rows, dense, lambdas, n_lambda, tol, max_sweeps, stall, support_dev,
+                          &res);
+        if (rc != CONCORD_OK) return rc;
+        total_ms += bt->last_ms;
+        for (size_t i = 0; i < dense.size(); ++i) {
+          const Item& it = dense[i];
+          const int code = take(it, it.k0, before[i], true);
+          if (code == 4 && brk)
+            pol.push_back({it.b, it.k0, 1, 0, 0});
+          else if (code != 2 && code != 3)
+            next[it.b] = it.k0 + 1;
+        }
       }
     }
-    if (pol.empty()) break;
-    for (const Item& it : pol)
-      if ((rc = promote(bt, bt->probs[it.b])) != CONCORD_OK) return rc;
-    rc = run_waves<double>(bt, rows, pol, lambdas, n_lambda, tol, max_sweeps, 0, nullptr, &res);
-    if (rc != CONCORD_OK) return rc;
-    total_ms += bt->last_ms;
-    for (const Item& it : pol) {
-      Prob& q = bt->probs[it.b];
-      if ((rc = demote(bt, q)) != CONCORD_OK) return rc;
-      if (support_dev)
-        BCK(launch_support_add(q.Om64, 0, q.ld, q.p, support_dev + (size_t)it.k0 * q.p * q.p,
-                               bt->stream));
-      const size_t o = ((size_t)it.b * n_lambda + it.k0) * kRes;
-      const double* x = res.data() + o;
-      const double s32 = (*R)[o + kResSweeps];
-      for (int q2 = 0; q2 < kRes; ++q2) (*R)[o + q2] = x[q2];
-      (*R)[o + kResSweeps] = s32 + x[kResSweeps];
-      next[it.b] = it.k0 + 1;
+    if (!pol.empty()) {
+      for (Item& it : pol) {
+        const int done = log->sweeps32[(size_t)it.b * n_lambda + it.k0];
+        it.n_sweeps = max_sweeps > done ? max_sweeps - done : 1;
+        if ((rc = promote(bt, bt->probs[it.b])) != CONCORD_OK) return rc;
+      }
+      rc = run_waves<double>(bt, rows, pol, lambdas, n_lambda, tol, max_sweeps, 0, nullptr, &res);
+      if (rc != CONCORD_OK) return rc;
+      total_ms += bt->last_ms;
+      for (const Item& it : pol) {
+        Prob& q = bt->probs[it.b];
+        if ((rc = demote(bt, q)) != CONCORD_OK) return rc;
+        if (support_dev)
+          BCK(launch_support_add(q.Om64, 0, q.ld, q.p, support_dev + (size_t)it.k0 * q.p * q.p,
+                                 bt->stream));
+        const size_t o = (size_t)it.b * n_lambda + it.k0;
+        const double* x = res.data() + o * kRes;
+        const double s32 = log->rows[o * kRes + kResSweeps];
+        for (int q2 = 0; q2 < kRes; ++q2) log->rows[o * kRes + q2] = x[q2];
+        log->rows[o * kRes + kResSweeps] = s32 + x[kResSweeps];
+        log->dense[o] += (int)x[kResSweeps];
+        next[it.b] = it.k0 + 1;
+      }
     }
   }
   BCK(cudaStreamSynchronize(bt->stream));
@@ -410,12 +597,13 @@ int mixed_path(concord_batch* bt, int rows, const double* lambdas, int n_lambda,
   return CONCORD_OK;
 }
 
-void fill_results(const std::vector<double>& r, const std::vector<int>* sweeps32, int B,
-                  int n_lambda, const double* lambdas, concord_result* out) {
+void fill_results(const PathLog& log, bool mixed, int B, int n_lambda, const double* lambdas,
+                  concord_result* out) {
   for (int b = 0; b < B; ++b)
     for (int k = 0; k < n_lambda; ++k) {
-      const double* x = r.data() + ((size_t)b * n_lambda + k) * kRes;
-      concord_result& o = out[(size_t)b * n_lambda + k];
+      const size_t c = (size_t)b * n_lambda + k;
+      const double* x = log.rows.data() + c * kRes;
+      concord_result& o = out[c];
       memset(&o, 0, sizeof o);
       const int code = (int)x[kResStatus];
       o.status = code == 0 ? CONCORD_OK
@@ -431,8 +619,9 @@ void fill_results(const std::vector<double>& r, const std::vector<int>* sweeps32
       o.active_pairs = (long long)(x[kResActive] + 0.5);
       o.timeout_vertex = -1;
       o.timeout_step = -1;
-      o.dense_sweeps = o.sweeps;
-      if (sweeps32) o.sweeps_fp32 = (*sweeps32)[(size_t)b * n_lambda + k];
+      o.screen_redos = (int)x[kResRedo];
+      o.dense_sweeps = log.dense[c];
+      if (mixed) o.sweeps_fp32 = log.sweeps32[c];
     }
 }
 
@@ -495,6 +684,7 @@ int concord_batch_create(concord_batch** out, int n_problems, const int* p, int 
     BALLOC(q.partials, sizeof(double) * kParts * (size_t)ctas_for(q.p, 2));
     BALLOC(q.mbox, sizeof(unsigned long long) * 2 * (size_t)kDepth * q.pe);
     BALLOC(q.barrier, sizeof(unsigned));
+    BALLOC(q.mrow, sizeof(float) * q.p);
     if (e == 4) {
       const size_t mat64 = sizeof(double) * (size_t)q.p * q.ld;
       BALLOC(q.S64, mat64);
@@ -521,6 +711,8 @@ int concord_batch_create(concord_batch** out, int n_problems, const int* p, int 
       BALLOC(bt->zt_lo, sizeof(float) * (size_t)n_pad * p_pad);
     } else {
       BALLOC(bt->Z, sizeof(double) * (size_t)n_cap * rup(bt->pmax, kTile));
+      if (gram_f64_bytes(n_cap, bt->pmax) > 0)
+        BALLOC(bt->gf_work, gram_f64_bytes(n_cap, bt->pmax));
     }
   }
 #undef BALLOC
@@ -578,6 +770,8 @@ int concord_batch_set_rows_per_warp(concord_batch* bt, int rows) {
   if (rows != 0 && rows != 2 && rows != 4 && rows != 8 && rows != 16 && rows != 32)
     return bfail(CONCORD_E_ARG, "rows per warp must be 0 (autotune), 2, 4, 8, 16 or 32");
   bt->rows_per_warp = rows;
+  bt->rows_set = rows > 0;
+  bt->reset_next = rows == 0;
   return CONCORD_OK;
 }
 
@@ -633,9 +827,9 @@ int concord_batch_gram(concord_batch* bt, int b, const void* X_dev, int x_dtype,
     BCK(launch_convert(X_dev, x_f32, ldx, bt->Xg, 0, p, nr, p, s));
   }
   BCK(cudaMemsetAsync(bt->flag, 0, sizeof(int), s));
-  BCK(launch_col_stats_chunked(bt->Xg, 0, nr, p, p, prep, bt->mean, bt->inv, bt->flag, bt->part,
-                               s));
   if (is_mixed(bt)) {
+    BCK(launch_col_stats_chunked(bt->Xg, 0, nr, p, p, prep, bt->mean, bt->inv, bt->flag, bt->part,
+                                 s));
     const int n_pad = rup(nr, 32), p_pad = rup(p, 128);
     BCK(launch_split_tf32(bt->Xg, 0, nr, p, p, bt->mean, bt->inv, bt->zt_hi, bt->zt_lo, n_pad,
                           p_pad, s));
@@ -643,19 +837,43 @@ int concord_batch_gram(concord_batch* bt, int b, const void* X_dev, int x_dtype,
                                        1.0f / nr, bt->flag, s);
     if (e == cudaErrorNotSupported) return bfail(CONCORD_E_CUDA, "tensor-core Gram unavailable");
     BCK(e);
-    BCK(launch_convert(q.S, 1, q.ld, q.S64, 0, q.ld, p, p, s));
+    // the FP64 copy and the starting iterate in one pass over S (checks in
+    // bits 8 and 16 of the same word, read once)
+    ResetMixedArgs ra;
+    memset(&ra, 0, sizeof ra);
+    ra.S = (const float*)q.S;
+    ra.ld = q.ld;
+    ra.p = p;
+    ra.P = q.P;
+    ra.W = (float*)q.W;
+    ra.Om = (float*)q.Om;
+    ra.S64 = q.S64;
+    ra.mrow = q.mrow;
+    ra.sdiag64 = q.sdiag64;
+    ra.sdiag32 = (float*)q.sdiagT;
+    ra.sd1 = (float*)q.sd1;
+    ra.sd2 = (float*)q.sd2;
+    ra.sd1_64 = q.sd1_64;
+    ra.sd2_64 = q.sd2_64;
+    ra.omdiag64 = q.omdiag64;
+    ra.bad = bt->flag;
+    BCK(launch_reset_mixed(ra, s));
   } else {
-    const int ldz = rup(p, kTile);
-    BCK(launch_apply_prep(bt->Xg, 0, nr, p, p, bt->mean, bt->inv, bt->Z, 0, ldz, s));
-    BCK(launch_syrk_f64((const double*)bt->Z, nr, p, ldz, (double*)q.S, q.ld, 1.0 / nr, s));
+    BCK(launch_gram_f64({bt->Xg, 0, nr, p, p, prep, bt->mean, bt->inv, bt->flag, bt->part,
+                         (double*)bt->Z, rup(p, kTile), bt->gf_work, (double*)q.S, q.ld}, s));
   }
   BCK(cudaMemcpyAsync(bt->h_flag, bt->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   BCK(cudaStreamSynchronize(s));
   const int bad = *bt->h_flag;
+  if (bad != 0) q.have_S = false;
   if (bad & 4) return bfail(CONCORD_E_TIMEOUT, "tensor-core Gram: a device-side wait ran out");
   if (bad & 2) return bfail(CONCORD_E_NONFINITE, "X has a non-finite entry");
   if (bad & 1) return bfail(CONCORD_E_NONPOS_DIAG, "X has a constant column");
-  return reset_prob(bt, q);
+  if (bad & 8) return bfail(CONCORD_E_NONFINITE, "S has a non-finite diagonal entry");
+  if (bad & 16) return bfail(CONCORD_E_NONPOS_DIAG, "S has a non-positive diagonal entry");
+  if (!is_mixed(bt)) return reset_prob(bt, q);
+  q.have_S = true;
+  return CONCORD_OK;
 }
 
 int concord_batch_reset(concord_batch* bt, int b) {
@@ -691,6 +909,7 @@ int concord_batch_autotune(concord_batch* bt, double lambda, int sweeps, double*
   }
   if (best == 0) return bfail(CONCORD_E_OCCUPANCY, "no rows-per-warp choice could launch");
   bt->rows_per_warp = best;
+  bt->rows_set = false;
   return CONCORD_OK;
 }
 
@@ -710,30 +929,17 @@ int concord_batch_path(concord_batch* bt, const double* lambdas, int n_lambda, d
     return bfail(CONCORD_E_ARG, "n_lambda x max_sweeps x p must stay below 2^31");
   BCK(cudaSetDevice(bt->device));
   int rc;
-  if (bt->rows_per_warp == 0) {
-    // autotune on a short run at the path's middle lambda, then start over
-    std::vector<double> ms(5);
-    if ((rc = concord_batch_autotune(bt, lambdas[n_lambda / 2], 2, ms.data())) != CONCORD_OK)
-      return rc;
-  }
-  std::vector<double> res;
-  if (is_mixed(bt) && bt->polish) {
-    std::vector<int> s32;
-    rc = mixed_path(bt, bt->rows_per_warp, lambdas, n_lambda, tol, max_sweeps, support_dev, &res,
-                    &s32);
-    if (rc != CONCORD_OK) return rc;
-    if (results) fill_results(res, &s32, (int)bt->probs.size(), n_lambda, lambdas, results);
-    return CONCORD_OK;
-  }
-  rc = run_any(bt, bt->rows_per_warp, lambdas, n_lambda, tol, max_sweeps, support_dev, &res);
+  if (bt->reset_next && !bt->rows_set)
+    for (auto& q : bt->probs)
+      if ((rc = reset_prob(bt, q)) != CONCORD_OK) return rc;
+  bt->reset_next = false;
+  PathLog log;
+  rc = is_mixed(bt)
+           ? walk<float>(bt, lambdas, n_lambda, tol, max_sweeps, support_dev, &log)
+           : walk<double>(bt, lambdas, n_lambda, tol, max_sweeps, support_dev, &log);
   if (rc != CONCORD_OK) return rc;
-  if (results) {
-    std::vector<int> s32;
-    if (is_mixed(bt))
-      for (size_t q = 0; q < res.size() / kRes; ++q) s32.push_back((int)res[q * kRes + kResSweeps]);
-    fill_results(res, is_mixed(bt) ? &s32 : nullptr, (int)bt->probs.size(), n_lambda, lambdas,
-                 results);
-  }
+  if (results)
+    fill_results(log, is_mixed(bt), (int)bt->probs.size(), n_lambda, lambdas, results);
   return CONCORD_OK;
 }
 

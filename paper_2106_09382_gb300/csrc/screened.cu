@@ -1819,7 +1819,14 @@ __global__ void __launch_bounds__(kScreenThreads, 1)
   for (int e = threadIdx.x; e < (int)(sizeof(ScreenArgs<T>) / sizeof(int)); e += blockDim.x)
     reinterpret_cast<int*>(&s_a)[e] = __ldg(src + e);
   __syncthreads();
-  screened_body<T, MIXED, true>(s_a, size, (int)(blockIdx.x % size));
+  // the counters a launch from scratch starts from
+  const int cta = (int)(blockIdx.x % size), step = size * (int)blockDim.x;
+  const int first = cta * (int)blockDim.x + (int)threadIdx.x;
+  for (int e = first; e < kCtrs; e += step) s_a.w.ctr[e] = 0;
+  for (int e = first; e <= s_a.p; e += step) s_a.w.cnt_r[0][e] = s_a.w.cnt_r[1][e] = 0;
+  for (int e = first; e < s_a.p; e += step) s_a.w.pend_n[e] = 0;
+  cluster_barrier();
+  screened_body<T, MIXED, true>(s_a, size, cta);
 }
 
 template <typename T, bool MIXED>

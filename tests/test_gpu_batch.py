@@ -187,3 +187,50 @@ def test_mixed_batch_without_polish_reports_the_stall():
         bt.set_S(0, dev(S))
         res = bt.path([0.3, 0.2], tol=1e-9, max_sweeps=2000)
     assert all(r.status == C.NOT_CONVERGED and r.sweeps < 2000 for r in res[0])
+
+
+@pytest.mark.parametrize("count,sizes", [(1, (2, 3)), (3, (31, 33, 64)), (20, (57, 100)), (90, (40,))])
+def test_screened_batch_is_bitwise_a_single_state_path(count, sizes):
+    """The default batch (one cluster per problem; 1 .. 90 problems, so
+    clusters of every size from one CTA up) ends every problem on the
+    single state's path iterate, bit for bit, in both precisions."""
+    lams = np.array([0.5, 0.3, 0.2])
+    ps = [sizes[b % len(sizes)] for b in range(count)]
+    Ss = [O.gram(O.standardize(data(2 * p + 20, p, 13 * p + b))) for b, p in enumerate(ps)]
+    for prec, dt in ((C.MIXED, torch.float32), (C.FP64, torch.float64)):
+        with C.Batch(ps, prec) as bt:
+            for b, S in enumerate(Ss):
+                bt.set_S(b, dev(S, dt))
+            res = bt.path(lams, tol=1e-5, max_sweeps=300)
+            G = [host(bt.get_omega(b, dt)) for b in range(count)]
+        for b in list(range(min(count, 4))) + [count - 1]:
+            with C.State(ps[b], prec) as st:
+                st.set_S(dev(Ss[b], dt))
+                ref = st.path(lams, tol=1e-5, max_sweeps=300)
+                assert np.array_equal(G[b], host(st.get_omega(dt)))
+                assert [r.sweeps for r in res[b]] == [r.sweeps for r in ref]
+
+
+def test_screened_batch_hands_a_dense_lambda_over():
+    """A lambda at which most pairs change (and the next, which starts from its
+    Omega) overflows a batched problem's lists of 16384 of the 44850 pairs: it
+    runs on the dense kernel, the walk resumes screened, and the iterates stay
+    the dense layout's."""
+    S = O.gram(O.standardize(data(400, 300, 21)))
+    lams = np.array([0.3, 0.002, 0.25, 0.24])
+    out = []
+    for rows in (0, 8):
+        with C.Batch([300, 300], C.FP64) as bt:
+            if rows:
+                bt.set_rows_per_warp(rows)
+            for b in range(2):
+                bt.set_S(b, dev(S))
+            res = bt.path(lams, tol=1e-6, max_sweeps=400)
+            out.append(host(bt.get_omega(1)))
+            sweeps = [r.sweeps for r in res[1]]
+            dense = [r.dense_sweeps for r in res[1]]
+        if rows:
+            assert dense == sweeps
+        else:
+            assert dense[0] == 0 and 0 < dense[1] <= sweeps[1] and dense[3] == 0
+    assert np.array_equal(out[0], out[1])
