@@ -88,6 +88,8 @@ struct concord_state {
   int* flag = nullptr;
   unsigned long long* lmax = nullptr;
   unsigned tag_base = 1;
+  unsigned long long* words = nullptr;  // wave form's exchange words (allocated on first use)
+  unsigned wave_tag = 1;                // of its next sweep
   double timeout_s = 2.0;
   int fault_vertex = -1, fault_step = -1;
   int max_grid = 0;
@@ -234,7 +236,10 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   const bool layout_set = own && (st->sweep_variant == CONCORD_SWEEP_GRID ||
                                   st->sweep_variant == CONCORD_SWEEP_CLUSTER);
   // bandwidth: sweeps handed over by the screened kernel change most pairs;
-  // they take the grid layout with one row per warp (all SMs stream rows)
+  // in FP32 they take the wave form (p = 1000: 3.3 ms a sweep colour by
+  // colour), else the grid layout with one row per warp (all SMs stream rows)
+  const bool wave = bandwidth && mixed && sweep_wave_blocks(p) <= kWaveMaxBlocks &&
+                    sweep_wave_blocks(p) <= st->sms && st->max_ctas == 0;
   const int variant = bandwidth    ? CONCORD_SWEEP_GRID
                       : layout_set ? st->sweep_variant
                                    : (mixed ? CONCORD_SWEEP_CLUSTER : CONCORD_SWEEP_GRID);
@@ -277,6 +282,17 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
     R = (p + TW - 1) / TW;
   }
   if (R > 32) return fail(CONCORD_E_ARG, "p=%d needs %d rows per warp (max 32)", p, R);
+  if (wave) {
+    const size_t bytes = sizeof(unsigned long long) * sweep_wave_words(p, 1);
+    if (!st->words) {
+      CK(cudaMalloc((void**)&st->words, bytes));
+      st->wave_tag = 0x80000000u;
+    }
+    if (st->wave_tag + (unsigned)n_sweeps >= 0x80000000u) {
+      CK(cudaMemsetAsync(st->words, 0, bytes, st->stream));
+      st->wave_tag = 1;
+    }
+  }
   st->last_variant = cluster ? CONCORD_SWEEP_CLUSTER : CONCORD_SWEEP_GRID;
 
   // keep step tags monotone over the state's lifetime; restart them (and
@@ -328,7 +344,8 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   a.stop_rule = stop_rule;
   a.n_sweeps = n_sweeps;
   a.kkt_only = kkt_only;
-  a.tag_base = st->tag_base;
+  a.tag_base = wave ? st->wave_tag : st->tag_base;
+  a.words = st->words;
   a.fault_vertex = st->fault_vertex;
   a.fault_step = st->fault_step;
   st->fault_vertex = -1;  // one-shot
@@ -336,9 +353,19 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
 
   const int slot_ev = st->n_launch < kMaxTimedLaunches ? st->n_launch : -1;
   if (slot_ev >= 0) CK(cudaEventRecord(st->lev[2 * slot_ev], st->stream));
-  CK(launch_sweep(a, grid, block, cluster, st->stream));
+  if constexpr (sizeof(T) == 4) {
+    if (wave) {
+      CK(launch_sweep_wave(a, st->sms, st->stream));
+      st->wave_tag += (unsigned)n_sweeps;
+    } else {
+      CK(launch_sweep(a, grid, block, cluster, st->stream));
+      st->tag_base += (unsigned)span;
+    }
+  } else {
+    CK(launch_sweep(a, grid, block, cluster, st->stream));
+    st->tag_base += (unsigned)span;
+  }
   if (slot_ev >= 0) CK(cudaEventRecord(st->lev[2 * slot_ev + 1], st->stream));
-  st->tag_base += (unsigned)span;
 
   CK(cudaMemcpyAsync(st->h_result, st->result, kRes * sizeof(double), cudaMemcpyDeviceToHost,
                      st->stream));
@@ -1397,7 +1424,7 @@ int concord_destroy(concord_state* st) {
                  st->hist, st->result, st->mean, st->inv_scale, st->Z, st->Xstage, st->zt_hi,
                  st->zt_lo, st->sdiag64, st->sdiagT, st->omdiag64, st->S64, st->W64, st->Om64,
                  st->zt32, st->rf.cnt, st->rf.off, st->rf.cur, st->rf.nbr, st->rf.ctr, st->rf.cand,
-                 st->rf.bitmap, st->mrow, st->pol.mem, st->gf_work};
+                 st->rf.bitmap, st->mrow, st->pol.mem, st->gf_work, st->words};
   for (void* d : dev)
     if (d) cudaFree(d);
   void* adj_dev[] = {st->adj.cnt, st->adj.rowptr, st->adj.bad, st->adj.col, st->adj.erow,

@@ -64,6 +64,7 @@ struct Prob {
   double *S64 = nullptr, *W64 = nullptr, *Om64 = nullptr, *sd1_64 = nullptr, *sd2_64 = nullptr;
   unsigned long long* mbox = nullptr;
   unsigned* barrier = nullptr;
+  unsigned long long* words = nullptr;  // wave form's exchange words (allocated on first use)
   float* mrow = nullptr;  // [p] m[u] >= max_{x != u} |s_ux| (lazy verification bound)
   // screened sweeps (allocated on first use): W after the sweep, W at each
   // pair's visit, the lists, per-CTA partial sums and the launch's result
@@ -86,6 +87,7 @@ struct concord_batch {
   std::vector<Prob> probs;
   double timeout_s = 2.0;
   int rows_per_warp = 0;  // dense layout; 0: not chosen
+  bool tuning = false;    // concord_batch_autotune is timing layouts
   bool reset_next = false;  // the layout was given back: the next path starts from Omega = I
   bool rows_set = false;  // chosen by the caller: every sweep runs on the dense kernel
   bool polish = true;     // MIXED: FP64 polish of a lambda whose FP32 sweeps stall
@@ -118,7 +120,7 @@ size_t esz(const concord_batch* bt) { return is_mixed(bt) ? 4 : 8; }
 void free_prob(Prob& q) {
   void* d[] = {q.S,        q.W,      q.Om,     q.sdiagT, q.sd1,    q.sd2,  q.sdiag64,
                q.omdiag64, q.partials, q.mbox, q.barrier, q.S64, q.W64, q.Om64,
-               q.sd1_64,   q.sd2_64, q.mrow, q.Wb, q.V, q.scr, q.sres};
+               q.sd1_64,   q.sd2_64, q.mrow, q.Wb, q.V, q.scr, q.sres, q.words};
   for (void* x : d)
     if (x) cudaFree(x);
   q = Prob();
@@ -222,9 +224,14 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
   int occ = 0;
   BCK(sweep_occupancy(sizeof(T) == 4, kSweepThreads, &occ));
   if (occ < 1) return bfail(CONCORD_E_OCCUPANCY, "sweep kernel cannot be resident");
-  const int capacity = bt->sms * occ;
+  // FP32 without a chosen layout: the wave form, one CTA per 32 rows
+  bool wave = sizeof(T) == 4 && !bt->rows_set && !bt->tuning;
   for (const auto& it : items)
-    if (ctas_for(bt->probs[it.b].p, rows) > capacity)
+    wave = wave && sweep_wave_blocks(bt->probs[it.b].p) <= std::min(kWaveMaxBlocks, bt->sms);
+  auto ctas_of = [&](int p) { return wave ? sweep_wave_blocks(p) : ctas_for(p, rows); };
+  const int capacity = wave ? bt->sms : bt->sms * occ;
+  for (const auto& it : items)
+    if (ctas_of(bt->probs[it.b].p) > capacity)
       return bfail(CONCORD_E_ARG, "p=%d needs more than %d CTAs at %d rows per warp",
                    bt->probs[it.b].p, capacity, rows);
   // device copies of the lambdas, the result rows and the problem table
@@ -236,7 +243,7 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
   {
     int i0 = 0, used = 0;
     for (int i = 0; i < nI; ++i) {
-      const int c = ctas_for(bt->probs[items[i].b].p, rows);
+      const int c = ctas_of(bt->probs[items[i].b].p);
       if (used + c > capacity && i > i0) {
         waves.push_back({i0, i});
         i0 = i;
@@ -258,7 +265,7 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
       e.P = q.P;
       e.ld = q.ld;
       e.cta0 = cta0;
-      e.ctas = ctas_for(q.p, rows);
+      e.ctas = ctas_of(q.p);
       cta0 += e.ctas;
       e.W = (T*)(copies ? (void*)q.W64 : q.W);
       e.Om = (T*)(copies ? (void*)q.Om64 : q.Om);
@@ -278,7 +285,14 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
       e.stall_break = it.stall_break;
       e.n_sweeps = it.n_sweeps;
       // fresh mailboxes: this launch's step tags start at 1
-      BCK(cudaMemsetAsync(q.mbox, 0, sizeof(unsigned long long) * 2 * (size_t)kDepth * q.pe, s));
+      if (wave) {
+        const size_t bytes = sizeof(unsigned long long) * sweep_wave_words(q.p, 1);
+        if (!q.words) BCK(cudaMalloc((void**)&q.words, bytes));
+        BCK(cudaMemsetAsync(q.words, 0, bytes, s));
+        e.words = q.words;
+      } else {
+        BCK(cudaMemsetAsync(q.mbox, 0, sizeof(unsigned long long) * 2 * (size_t)kDepth * q.pe, s));
+      }
       BCK(cudaMemsetAsync(q.barrier, 0, sizeof(unsigned), s));
     }
   }
@@ -316,7 +330,11 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
     int grid = 0;
     for (int i = w.first; i < w.second; ++i) grid += table[i].ctas;
     total_ctas = std::max(total_ctas, grid);
-    BCK(launch_sweep_batch(a, grid, kSweepThreads, s));
+    if constexpr (sizeof(T) == 4) {
+      BCK(wave ? launch_sweep_wave_batch(a, grid, s) : launch_sweep_batch(a, grid, kSweepThreads, s));
+    } else {
+      BCK(launch_sweep_batch(a, grid, kSweepThreads, s));
+    }
   }
   BCK(cudaEventRecord(bt->ev1, s));
   res_host->assign(nres, 0.0);
@@ -895,7 +913,9 @@ int concord_batch_autotune(concord_batch* bt, double lambda, int sweeps, double*
   int i = 0;
   for (int rows : kRowsChoices) {
     std::vector<double> res;
+    bt->tuning = true;
     int rc = run_any(bt, rows, &lambda, 1, -1.0, sweeps, nullptr, &res);
+    bt->tuning = false;
     float ms = rc == CONCORD_OK ? bt->last_ms : -1.f;
     if (ms_per_choice) ms_per_choice[i] = ms;
     ++i;

@@ -23,6 +23,7 @@
 
 #include "joint.h"
 #include "kernels.h"
+#include "wave.cuh"
 
 namespace concord {
 namespace {
@@ -248,8 +249,41 @@ __device__ __forceinline__ void warp_axpy(T* __restrict__ w, const T* __restrict
   }
 }
 
+// A sweep's blocks in the wave form.
+struct WaveJoint {
+  const JointArgs<float>& a;
+  float l1, l2;
+  float dmax = 0.f;
+  int moved = 0;  // both owners count a pair
+  __device__ void pair(const float (&c)[2], const float (&om)[2], const float (&wa)[2],
+                       const float (&wb)[2], float (&nw)[2]) {
+    const float g1 = (wa[0] + wb[0]) - c[0] * om[0];
+    const float g2 = (wa[1] + wb[1]) - c[1] * om[1];
+    block_pair<float>(c[0], g1, c[1], g2, l1, l2, nw[0], nw[1]);
+  }
+  __device__ void count(const float (&d)[2]) {
+    dmax = nmax<float>(dmax, nmax<float>(fabsf(d[0]), fabsf(d[1])));
+    if (d[0] != 0.f || d[1] != 0.f) ++moved;
+  }
+  __device__ void diag(int i, const float (&w)[2], float (&dd)[2]) {
+    const size_t ii = (size_t)i * a.ld + i;
+    const float o1 = a.Om[0][ii], o2 = a.Om[1][ii];
+    const float s1 = __ldg(a.S[0] + ii), s2 = __ldg(a.S[1] + ii);
+    const float b1 = w[0] - o1 * s1;
+    const float b2 = w[1] - o2 * s2;
+    float n1, n2;
+    block_diag<float>(s1, b1, s2, b2, l2, n1, n2);
+    dd[0] = n1 - o1;
+    dd[1] = n2 - o2;
+    if (dd[0] != 0.f) a.Om[0][ii] = n1;
+    if (dd[1] != 0.f) a.Om[1][ii] = n2;
+    dmax = nmax<float>(dmax, nmax<float>(fabsf(dd[0]), fabsf(dd[1])));
+  }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
   const int p = a.p, P = a.P, ld = a.ld;
   const int half = (P + 1) / 2;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -274,7 +308,35 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
     const bool swept = !initial && t < a.n_sweeps;
     T dmax = (T)0;  // lane-0 / thread-local contributions, kept in T (FP64 is slow here)
     int moved = 0;
-    if (swept) {
+    bool tiled = false;  // this sweep ran in the wave form
+    if constexpr (sizeof(T) == 4) {
+      if (swept && a.words != nullptr) {
+        tiled = true;
+        if ((int)blockIdx.x < wave_blocks(p)) {
+          WaveArgs<2> wa;
+          wa.p = p;
+          wa.P = P;
+          wa.ld = ld;
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            wa.S[m] = a.S[m];
+            wa.W[m] = a.W[m];
+            wa.Om[m] = a.Om[m];
+            wa.sdiag[m] = a.S[m];
+          }
+          wa.sd_stride = (size_t)ld + 1;
+          wa.words = a.words;
+          wa.tag = a.tag + (unsigned)t;
+          wa.wait = a.wait;
+          WaveJoint ops{a, l1t, l2t};
+          wave_sweep<2>(wa, *reinterpret_cast<WaveSmem<2>*>(dyn), (int)blockIdx.x, ops);
+          dmax = ops.dmax;
+          moved = ops.moved;
+        }
+        grid_barrier(a.barrier, gen, a.wait, P);
+      }
+    }
+    if (swept && !tiled) {
       // ---- colour steps
       for (int c = 0; c < P; ++c) {
         for (int base = blockIdx.x * kJointWarps; base < half; base += gridDim.x * kJointWarps) {
@@ -416,7 +478,7 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
       for (int e = threadIdx.x; e < 2 * 1024; e += blockDim.x) {
         const int m = e >> 10, r = (e >> 5) & 31, c = e & 31;
         const int row = 32 * bj + r;
-        wt[m][c][r] = row < p ? a.W[m][(size_t)row * ld + 32 * bi + c] : (T)0;
+        wt[m][c][r] = row < p ? __ldcg(a.W[m] + (size_t)row * ld + 32 * bi + c) : (T)0;
       }
       __syncthreads();
       for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
@@ -424,8 +486,8 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
         const int i = 32 * bi + ty, j = 32 * bj + tx;
         if (i >= p || j >= p || i > j) continue;
         const size_t ij = (size_t)i * ld + j;
-        const T x = a.Om[0][ij], y = a.Om[1][ij];
-        const T wa = a.W[0][ij], wb = a.W[1][ij];
+        const T x = __ldcg(a.Om[0] + ij), y = __ldcg(a.Om[1] + ij);
+        const T wa = __ldcg(a.W[0] + ij), wb = __ldcg(a.W[1] + ij);
         if (i == j) {
           const T ga = wa - (T)1 / x, gb = wb - (T)1 / y;
           kk = nmax<T>(kk, diag_kkt<T>(ga, gb, x, y, l2t));
@@ -445,7 +507,7 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
     // block reduction of the partials
     {
       double v[kJParts] = {(double)kk, (double)quad, (double)logs, (double)pen, (double)fuse,
-                           (double)dmax, (double)moved, 0.0};
+                           (double)dmax, tiled ? 0.5 * (double)moved : (double)moved, 0.0};
 #pragma unroll
       for (int q = 0; q < kJParts; ++q) {
         double x = v[q];
@@ -582,8 +644,15 @@ cudaError_t launch_joint_t(const JointArgs<T>& a, int grid, cudaStream_t st) {
   if (a.ld % 32 != 0 || a.p < 2 || grid < 1) return cudaErrorInvalidValue;
   void* args[] = {(void*)&a};
   note_launches(1);
+  const size_t dyn = sizeof(T) == 4 && a.words != nullptr ? sizeof(WaveSmem<2>) : 0;
+  if (dyn > 0) {
+    if (grid < wave_blocks(a.p)) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_joint<T>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    if (e != cudaSuccess) return e;
+  }
   return cudaLaunchCooperativeKernel((const void*)k_joint<T>, dim3(grid), dim3(kJointThreads),
-                                     args, 0, st);
+                                     args, dyn, st);
 }
 
 }  // namespace
@@ -594,6 +663,10 @@ cudaError_t launch_joint(const JointArgs<double>& a, int grid, cudaStream_t st) 
 cudaError_t launch_joint(const JointArgs<float>& a, int grid, cudaStream_t st) {
   return launch_joint_t(a, grid, st);
 }
+
+int joint_wave_blocks(int p) { return wave_blocks(p); }
+size_t joint_wave_words(int p) { return wave_words(p, 2); }
+static_assert(kWaveThreads == kJointThreads, "the wave form runs in the joint kernel's CTAs");
 
 cudaError_t joint_occupancy(bool f32, int* blocks_per_sm) {
   return f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_joint<float>,

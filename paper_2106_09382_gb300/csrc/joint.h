@@ -51,12 +51,18 @@ struct JointArgs {
   double* hist;              // hist_len x kJHist
   int hist_len;
   double* result;            // kJRes
+  unsigned long long* words; // FP32: exchange words of the wave form (wave.cuh), or nullptr:
+                             // colour by colour
+  unsigned tag;              // of the launch's first sweep
 };
 
 // One persistent cooperative launch (grid CTAs of kJointThreads threads,
 // co-resident): joint sweeps until the stopping rule or n_sweeps.
 cudaError_t launch_joint(const JointArgs<double>& a, int grid, cudaStream_t st);
 cudaError_t launch_joint(const JointArgs<float>& a, int grid, cudaStream_t st);
+// With a.words the grid has at least joint_wave_blocks(p) CTAs.
+int joint_wave_blocks(int p);
+size_t joint_wave_words(int p);
 cudaError_t joint_occupancy(bool f32, int* blocks_per_sm);
 
 // W (p x ld) = Om S, skipping the zero entries of each row of Om (one warp per

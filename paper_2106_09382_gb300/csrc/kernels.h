@@ -65,6 +65,7 @@ struct BatchProblem {
   double* result;            // nk x kRes: the result of each lambda it walks
   float* cnt;                // nullable: slice k (p x p) += [w_ij != 0] after its lambda k
   int k0, nk;                // it walks lambdas[k0 .. k0 + nk)
+  unsigned long long* words; // wave form: exchange words (zeroed before the launch)
   int stall_break;           // a lambda that ends on the stall rule ends the problem's walk
   int n_sweeps;              // > 0: its sweep limit per lambda (else the launch's)
 };
@@ -95,6 +96,7 @@ struct SweepArgs {
   unsigned poll_ns;          // back-off between mailbox polls (0: none)
   unsigned tag_base;
   int fault_vertex, fault_step;
+  unsigned long long* words;  // wave form: exchange words (wave.cuh); tags from tag_base
   // batched launch (launch_sweep_batch): problems and the lambda path every
   // problem walks (warm-started, n_sweeps sweeps at most per lambda)
   const BatchProblem<T>* probs;
@@ -119,6 +121,15 @@ cudaError_t sweep_occupancy(bool mixed, int block, int* blocks_per_sm);
 // the abort word and nothing else.
 cudaError_t launch_sweep_batch(const SweepArgs<double>& a, int grid, int block, cudaStream_t st);
 cudaError_t launch_sweep_batch(const SweepArgs<float>& a, int grid, int block, cudaStream_t st);
+// The wave form (FP32, wave.cuh): tiles of 32 x 32 vertices instead of colour
+// steps, one CTA per block of 32 rows; the same iterates.  launch_sweep_wave:
+// grid >= wave_blocks(p) CTAs (the others join the KKT pass).  _batch: as
+// launch_sweep_batch, wave_blocks(p) CTAs per problem.
+constexpr int kWaveMaxBlocks = 64;  // the exchange words grow with the square (35 MB here)
+cudaError_t launch_sweep_wave(const SweepArgs<float>& a, int grid, cudaStream_t st);
+cudaError_t launch_sweep_wave_batch(const SweepArgs<float>& a, int grid, cudaStream_t st);
+int sweep_wave_blocks(int p);
+size_t sweep_wave_words(int p, int matrices);
 // Largest launchable cluster (power of two <= 16; 0 if none).
 cudaError_t sweep_cluster_size(bool mixed, int block, int row_warps, int rows_per_warp, int* cs);
 

@@ -21,6 +21,7 @@
 //     KKT / objective pass; a second one publishes its partial results.
 #include "common.cuh"
 #include "kernels.h"
+#include "wave.cuh"
 
 namespace concord {
 
@@ -223,6 +224,8 @@ __device__ __forceinline__ bool box_read<double>(const unsigned long long* local
 //     word a row reads lives in its own CTA's shared memory and the partner
 //     stores into it through distributed shared memory (lower latency), with
 //     per-row progress counters guarding slot reuse.
+//   WAVE = true (FP32): a sweep runs tile by tile (wave.cuh) on the first
+//     wave_blocks(p) CTAs of the group; the others join the KKT pass.
 //   BATCH = true (grid form): the launch serves a.n_probs independent
 //     problems; each CTA belongs to one problem (its CTA range), whose rows,
 //     mailbox ring, barriers and partial sums are its own, and each problem
@@ -234,7 +237,38 @@ __device__ __forceinline__ const SweepArgs<T>& pick_args(const SweepArgs<T>& bat
   return use_batch ? batch : single;
 }
 
-template <typename T, bool MIXED, bool CLUSTER, bool BATCH>
+// A sweep's pairs and diagonal in the wave form.
+struct WaveSingle {
+  const SweepArgs<float>& A;
+  float lam;
+  float dpair = 0.f;   // largest change of a pair
+  double ddiag = 0.0;  // of a diagonal entry
+  int active = 0;
+  __device__ void pair(const float (&c)[1], const float (&om)[1], const float (&wa)[1],
+                       const float (&wb)[1], float (&nw)[1]) {
+    const float x = (c[0] * om[0] - wa[0]) - wb[0];
+    const float sx = soft_threshold(x, lam);
+    nw[0] = 0.f;
+    if (sx != 0.f) nw[0] = sx / c[0];
+  }
+  __device__ void count(const float (&d)[1]) {
+    if (d[0] != 0.f) {
+      dpair = fmaxf(dpair, fabsf(d[0]));
+      ++active;
+    }
+  }
+  __device__ void diag(int i, const float (&w)[1], float (&dd)[1]) {
+    const double sii = A.sdiag64[i], oii = A.omdiag64[i];
+    const double ci = (double)w[0] - oii * sii;
+    const double nw = (-ci + sqrt(ci * ci + 4.0 * sii)) / (2.0 * sii);
+    A.omdiag64[i] = nw;
+    A.Om[(size_t)i * A.ld + i] = (float)nw;
+    dd[0] = (float)(nw - oii);
+    ddiag = fmax(ddiag, fabs(nw - oii));
+  }
+};
+
+template <typename T, bool MIXED, bool CLUSTER, bool BATCH, bool WAVE = false>
 __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a) {
   using MB = Mailbox<T>;
   constexpr unsigned FULL = 0xffffffffu;
@@ -269,6 +303,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
       s_args.sdiag64 = q.sdiag64;
       s_args.omdiag64 = q.omdiag64;
       s_args.mbox = q.mbox;
+      s_args.words = q.words;
       s_args.barrier = q.barrier;
       s_args.partials = q.partials;
       s_args.result = q.result;
@@ -289,7 +324,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
     cta = s_gc[1];
   }
   const SweepArgs<T>& A = pick_args<T>(s_args, a, BATCH);
-  const bool row_warp = wid < A.row_warps;
+  const bool row_warp = WAVE || wid < A.row_warps;
   const int p = A.p, P = A.P, ld = A.ld;
   const int pe = P + 1;
   const int R = A.rows_per_warp;
@@ -300,10 +335,12 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
   int myrow;
   if constexpr (CLUSTER) {
     myrow = li * CS + (int)cta;
+  } else if constexpr (WAVE) {
+    myrow = lane < 2 ? cta * kWaveB + 2 * wid + lane : A.p;
   } else {
     myrow = (cta * A.row_warps + wid) + lane * (G * A.row_warps);
   }
-  const bool has_row = row_warp && lane < R && myrow < p;
+  const bool has_row = row_warp && (WAVE || lane < R) && myrow < p;
   // the lambda in force (batch: walks the path, index kl)
   double lam_cur = A.lambda;
   T lam = (T)lam_cur;
@@ -348,7 +385,26 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
   for (;;) {
     const bool do_sweep = !A.kkt_only && (BATCH ? t_lam : t) < A.n_sweeps;
     double dmax = 0.0, nact = 0.0;
-    if (do_sweep && row_warp) {
+    if constexpr (WAVE) {
+      if (do_sweep && cta < wave_blocks(p)) {
+        WaveArgs<1> wa;
+        wa.p = p;
+        wa.P = P;
+        wa.ld = ld;
+        wa.S[0] = A.S;
+        wa.W[0] = A.W;
+        wa.Om[0] = A.Om;
+        wa.sdiag[0] = A.sdiag;
+        wa.sd_stride = 1;
+        wa.words = A.words;
+        wa.tag = A.tag_base + (unsigned)t;
+        wa.wait = wc;
+        WaveSingle ops{A, lam};
+        wave_sweep<1>(wa, *reinterpret_cast<WaveSmem<1>*>(dyn), cta, ops);
+        dmax = fmax((double)ops.dpair, ops.ddiag);
+        nact = (double)ops.active;
+      }
+    } else if (do_sweep && row_warp) {
       const unsigned step0 = tag_base + (unsigned)(t * P);
       int cnt = 0;  // pending updates of this lane's row
       // Partners without integer division: for v >= 1 the ring index
@@ -847,9 +903,11 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
             const int i = __shfl_sync(FULL, myrow, k);
             const T* orow = A.Om + (size_t)i * ld;
             for (int x = lane; x < p; x += 32)
-              if (orow[x] != (T)0) atomicAdd(cnt_k + (size_t)i * p + x, 1.0f);
+              if (__ldcg(orow + x) != (T)0) atomicAdd(cnt_k + (size_t)i * p + x, 1.0f);
           }
         }
+        // (wave form: row 0 is written by every CTA of the group)
+        if (WAVE && A.batch_cnt && s_lam_count) group_barrier(A.barrier, gen, G, wc, 3000000 + t, cta);
         if (!s_stop) {
           ++kl;
           lam_cur = A.lambdas[kl];
@@ -967,6 +1025,28 @@ cudaError_t launch_sweep_batch(const SweepArgs<double>& a, int grid, int block, 
 cudaError_t launch_sweep_batch(const SweepArgs<float>& a, int grid, int block, cudaStream_t st) {
   return launch_sweep_batch_impl<float, true>(a, grid, block, st);
 }
+
+cudaError_t launch_sweep_wave(const SweepArgs<float>& args, int grid, cudaStream_t st) {
+  const size_t dyn = sizeof(WaveSmem<1>);
+  const void* fn = (const void*)k_sweep<float, true, false, false, true>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  note_launches(1);
+  void* kargs[] = {(void*)&args};
+  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveThreads), kargs, dyn, st);
+}
+cudaError_t launch_sweep_wave_batch(const SweepArgs<float>& args, int grid, cudaStream_t st) {
+  const size_t dyn = sizeof(WaveSmem<1>);
+  const void* fn = (const void*)k_sweep<float, true, false, true, true>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  note_launches(1);
+  void* kargs[] = {(void*)&args};
+  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveThreads), kargs, dyn, st);
+}
+int sweep_wave_blocks(int p) { return wave_blocks(p); }
+size_t sweep_wave_words(int p, int matrices) { return wave_words(p, matrices); }
+static_assert(kWaveThreads == kSweepThreads, "the wave form runs in the sweep kernel's CTAs");
 
 cudaError_t sweep_occupancy(bool mixed, int block, int* blocks_per_sm) {
   return mixed ? sweep_occupancy_impl<float, true>(block, blocks_per_sm)

@@ -273,3 +273,25 @@ def test_joint_fault_switch_arguments():
         J.set_fault(5, 2)  # ignored by the barrier variant
         r = J.run(0.1, 0.02, tol=1e-8, max_sweeps=500)
         assert r.status == C.OK
+
+
+@pytest.mark.parametrize("p", [2, 3, 31, 32, 33, 63, 64, 65, 97, 129, 200])
+def test_wave_form_is_bitwise_the_colour_by_colour_sweep(p):
+    """The FP32 sweeps' default (tiles of 32 x 32 vertices) against colour
+    steps on an explicit grid, sweep by sweep: block edges, ragged last
+    blocks, byes, tiles visited twice in a row."""
+    S1, S2 = grams(p, 3 * p + 20, p)
+    out = []
+    for grid in (0, 8):
+        with C.Joint(p, C.MIXED) as J:
+            if grid:
+                J.set_grid(grid)
+            J.set_S(0, dev(S1))
+            J.set_S(1, dev(S2))
+            rows = []
+            for n in (1, 3, 2):
+                r = J.sweep(0.05, 0.02, n)
+                rows += [r.delta, r.active_pairs] + [host(J.get_omega(m)) for m in (0, 1)]
+            out.append(rows)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)

@@ -151,3 +151,26 @@ def test_stability_workers_do_not_change_frequencies():
         f1 = host(st.stability(dev(X), subsets, lams, tol=1e-8, max_sweeps=1000, workers=1))
         f4 = host(st.stability(dev(X), subsets, lams, tol=1e-8, max_sweeps=1000, workers=4))
     assert np.array_equal(f1, f4)
+
+
+@pytest.mark.parametrize("p", [200, 225, 257, 416])
+def test_dense_lambdas_equal_the_dense_kernel_bit_for_bit(p):
+    """Lambdas at which most pairs change (the correction terms of p^2 / 2
+    candidates do not fit from p = 182 on) run in the wave form (FP32 tiles);
+    the path's iterates equal those of the dense grid kernel's sweeps."""
+    rng = np.random.default_rng(p)
+    X = rng.standard_normal((2 * p, p))
+    X[:, 1:] += 0.5 * X[:, :-1]
+    S = dev(O.gram(O.standardize(X)), torch.float32)
+    lams = [0.05, 0.001, 0.0005]
+    with C.State(p, C.MIXED) as st, C.Batch([p], C.MIXED) as bt:
+        st.set_S(S)
+        res = st.path(lams, tol=1e-12, max_sweeps=4)
+        bt.set_S(0, S)
+        bt.set_polish(False)
+        bt.set_rows_per_warp(4)  # every sweep colour by colour
+        ref = bt.path(lams, tol=1e-12, max_sweeps=4)[0]
+        assert [r.sweeps for r in res] == [r.sweeps for r in ref]
+        assert res[-1].dense_sweeps > 0
+        assert np.array_equal(host(st.get_omega(torch.float32)), host(bt.get_omega(0, torch.float32)))
+        assert res[-1].kkt == ref[-1].kkt
