@@ -238,7 +238,7 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   // bandwidth: sweeps handed over by the screened kernel change most pairs;
   // in FP32 they take the wave form (p = 1000: 3.3 ms a sweep colour by
   // colour), else the grid layout with one row per warp (all SMs stream rows)
-  const bool wave = bandwidth && mixed && sweep_wave_blocks(p) <= kWaveMaxBlocks &&
+  const bool wave = bandwidth && mixed && !kkt_only && sweep_wave_blocks(p) <= kWaveMaxBlocks &&
                     sweep_wave_blocks(p) <= st->sms && st->max_ctas == 0;
   const int variant = bandwidth    ? CONCORD_SWEEP_GRID
                       : layout_set ? st->sweep_variant
@@ -344,8 +344,7 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   a.stop_rule = stop_rule;
   a.n_sweeps = n_sweeps;
   a.kkt_only = kkt_only;
-  a.tag_base = wave ? st->wave_tag : st->tag_base;
-  a.words = st->words;
+  a.tag_base = st->tag_base;
   a.fault_vertex = st->fault_vertex;
   a.fault_step = st->fault_step;
   st->fault_vertex = -1;  // one-shot
@@ -355,7 +354,34 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   if (slot_ev >= 0) CK(cudaEventRecord(st->lev[2 * slot_ev], st->stream));
   if constexpr (sizeof(T) == 4) {
     if (wave) {
-      CK(launch_sweep_wave(a, st->sms, st->stream));
+      WaveLaunch w;
+      memset(&w, 0, sizeof w);
+      w.one.p = p;
+      w.one.P = st->P;
+      w.one.ld = st->ld;
+      w.one.ctas = sweep_wave_blocks(p);
+      w.one.W = W;
+      w.one.Om = Om;
+      w.one.S = S;
+      w.one.sdiag = sdiagT;
+      w.one.sdiag64 = st->sdiag64;
+      w.one.omdiag64 = omdiag64;
+      w.one.result = st->result;
+      w.one.nk = 1;
+      w.one.words = st->words;
+      w.lambda = lambda;
+      w.tol = tol;
+      w.delta_tol = a.delta_tol;
+      w.stop_rule = stop_rule;
+      w.n_sweeps = n_sweeps;
+      w.stall_stop = stall_stop;
+      w.tag0 = st->wave_tag;
+      w.wait = a.wait;
+      w.hist = a.hist;
+      w.hist_len = a.hist_len;
+      w.words0 = st->words;
+      w.p0 = p;
+      CK(run_sweep_wave(w, p, w.one.ctas, st->sms, false, st->stream));
       st->wave_tag += (unsigned)n_sweeps;
     } else {
       CK(launch_sweep(a, grid, block, cluster, st->stream));

@@ -327,11 +327,32 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
     a.n_probs = w.second - w.first;
     a.lambdas = bt->lam_dev;
     a.n_lambda = n_lambda;
-    int grid = 0;
-    for (int i = w.first; i < w.second; ++i) grid += table[i].ctas;
+    int grid = 0, p_max = 0;
+    for (int i = w.first; i < w.second; ++i) {
+      grid += table[i].ctas;
+      p_max = std::max(p_max, table[i].p);
+    }
     total_ctas = std::max(total_ctas, grid);
     if constexpr (sizeof(T) == 4) {
-      BCK(wave ? launch_sweep_wave_batch(a, grid, s) : launch_sweep_batch(a, grid, kSweepThreads, s));
+      if (wave) {
+        WaveLaunch l;
+        memset(&l, 0, sizeof l);
+        l.probs = a.probs;
+        l.n_probs = a.n_probs;
+        l.lambdas = a.lambdas;
+        l.tol = tol;
+        l.delta_tol = a.delta_tol;
+        l.stop_rule = a.stop_rule;
+        l.n_sweeps = max_sweeps;
+        l.stall_stop = stall_stop;
+        l.tag0 = 1;
+        l.wait = a.wait;
+        l.words0 = first.words;
+        l.p0 = first.p;
+        BCK(run_sweep_wave(l, p_max, grid, bt->sms, support_dev != nullptr, s));
+      } else {
+        BCK(launch_sweep_batch(a, grid, kSweepThreads, s));
+      }
     } else {
       BCK(launch_sweep_batch(a, grid, kSweepThreads, s));
     }

@@ -21,9 +21,11 @@
 //     triangle computes the joint KKT residual and the joint objective.
 #include <math.h>
 
+#include <algorithm>
+
 #include "joint.h"
-#include "kernels.h"
 #include "wave.cuh"
+#include "kernels.h"
 
 namespace concord {
 namespace {
@@ -249,41 +251,77 @@ __device__ __forceinline__ void warp_axpy(T* __restrict__ w, const T* __restrict
   }
 }
 
-// A sweep's blocks in the wave form.
-struct WaveJoint {
-  const JointArgs<float>& a;
-  float l1, l2;
-  float dmax = 0.f;
-  int moved = 0;  // both owners count a pair
-  __device__ void pair(const float (&c)[2], const float (&om)[2], const float (&wa)[2],
-                       const float (&wb)[2], float (&nw)[2]) {
-    const float g1 = (wa[0] + wb[0]) - c[0] * om[0];
-    const float g2 = (wa[1] + wb[1]) - c[1] * om[1];
-    block_pair<float>(c[0], g1, c[1], g2, l1, l2, nw[0], nw[1]);
-  }
-  __device__ void count(const float (&d)[2]) {
-    dmax = nmax<float>(dmax, nmax<float>(fabsf(d[0]), fabsf(d[1])));
-    if (d[0] != 0.f || d[1] != 0.f) ++moved;
-  }
-  __device__ void diag(int i, const float (&w)[2], float (&dd)[2]) {
-    const size_t ii = (size_t)i * a.ld + i;
-    const float o1 = a.Om[0][ii], o2 = a.Om[1][ii];
-    const float s1 = __ldg(a.S[0] + ii), s2 = __ldg(a.S[1] + ii);
-    const float b1 = w[0] - o1 * s1;
-    const float b2 = w[1] - o2 * s2;
-    float n1, n2;
-    block_diag<float>(s1, b1, s2, b2, l2, n1, n2);
-    dd[0] = n1 - o1;
-    dd[1] = n2 - o2;
-    if (dd[0] != 0.f) a.Om[0][ii] = n1;
-    if (dd[1] != 0.f) a.Om[1][ii] = n2;
-    dmax = nmax<float>(dmax, nmax<float>(fabsf(dd[0]), fabsf(dd[1])));
-  }
+// Largest residual and sums of a CTA's share of the upper-triangle tiles.
+template <typename T>
+struct JointSums {
+  T kk = (T)0, quad = (T)0, logs = (T)0, pen = (T)0, fuse = (T)0;
 };
+template <typename T>
+__device__ __forceinline__ void joint_pass(int p, int ld, const T* const (&W)[2], const T* const (&Om)[2],
+                                           T l1t, T l2t, int cta, int G, T (&wt)[2][32][33],
+                                           JointSums<T>& v) {
+  const int nt = (p + 31) / 32;
+  for (int k = cta; k < nt * nt; k += G) {
+    const int bi = k / nt, bj = k % nt;
+    if (bi > bj) continue;
+    // wt[m][c][r] = W_m[32 bj + r][32 bi + c]
+    for (int e = threadIdx.x; e < 2 * 1024; e += blockDim.x) {
+      const int m = e >> 10, r = (e >> 5) & 31, c = e & 31;
+      const int row = 32 * bj + r;
+      wt[m][c][r] = row < p ? __ldcg(W[m] + (size_t)row * ld + 32 * bi + c) : (T)0;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+      const int ty = e >> 5, tx = e & 31;
+      const int i = 32 * bi + ty, j = 32 * bj + tx;
+      if (i >= p || j >= p || i > j) continue;
+      const size_t ij = (size_t)i * ld + j;
+      const T x = __ldcg(Om[0] + ij), y = __ldcg(Om[1] + ij);
+      const T wa = __ldcg(W[0] + ij), wb = __ldcg(W[1] + ij);
+      if (i == j) {
+        const T ga = wa - (T)1 / x, gb = wb - (T)1 / y;
+        v.kk = nmax<T>(v.kk, diag_kkt<T>(ga, gb, x, y, l2t));
+        v.quad += x * wa + y * wb;
+        v.logs += log(x) + log(y);
+        v.fuse += fabs(x - y);
+      } else {
+        const T g1 = wa + wt[0][ty][tx], g2 = wb + wt[1][ty][tx];
+        v.kk = nmax<T>(v.kk, pair_kkt<T>(g1, g2, x, y, l1t, l2t));
+        v.quad += x * g1 + y * g2;
+        v.pen += fabs(x) + fabs(y);
+        v.fuse += fabs(x - y);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// out[k] = the block's partials (thread 0 .. kJParts - 1).
+__device__ __forceinline__ void joint_reduce(const double (&v)[kJParts], double (*red)[kJParts],
+                                             double* out) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int q = 0; q < kJParts; ++q) {
+    double x = v[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_down_sync(kFull, x, o);
+      x = (q == kJPartKkt || q == kJPartDelta) ? nmax<double>(x, y) : x + y;
+    }
+    if (lane == 0) red[wid][q] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < kJParts) {
+    const int q = threadIdx.x;
+    double x = red[0][q];
+    for (int w = 1; w < nw; ++w)
+      x = (q == kJPartKkt || q == kJPartDelta) ? nmax<double>(x, red[w][q]) : x + red[w][q];
+    out[q] = x;
+  }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char dyn[];
   const int p = a.p, P = a.P, ld = a.ld;
   const int half = (P + 1) / 2;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -308,35 +346,7 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
     const bool swept = !initial && t < a.n_sweeps;
     T dmax = (T)0;  // lane-0 / thread-local contributions, kept in T (FP64 is slow here)
     int moved = 0;
-    bool tiled = false;  // this sweep ran in the wave form
-    if constexpr (sizeof(T) == 4) {
-      if (swept && a.words != nullptr) {
-        tiled = true;
-        if ((int)blockIdx.x < wave_blocks(p)) {
-          WaveArgs<2> wa;
-          wa.p = p;
-          wa.P = P;
-          wa.ld = ld;
-#pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            wa.S[m] = a.S[m];
-            wa.W[m] = a.W[m];
-            wa.Om[m] = a.Om[m];
-            wa.sdiag[m] = a.S[m];
-          }
-          wa.sd_stride = (size_t)ld + 1;
-          wa.words = a.words;
-          wa.tag = a.tag + (unsigned)t;
-          wa.wait = a.wait;
-          WaveJoint ops{a, l1t, l2t};
-          wave_sweep<2>(wa, *reinterpret_cast<WaveSmem<2>*>(dyn), (int)blockIdx.x, ops);
-          dmax = ops.dmax;
-          moved = ops.moved;
-        }
-        grid_barrier(a.barrier, gen, a.wait, P);
-      }
-    }
-    if (swept && !tiled) {
+    if (swept) {
       // ---- colour steps
       for (int c = 0; c < P; ++c) {
         for (int base = blockIdx.x * kJointWarps; base < half; base += gridDim.x * kJointWarps) {
@@ -469,64 +479,12 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
 
     // ---- fused KKT / objective pass over the upper-triangle tiles
     // per-thread partials in T (a few dozen terms each), combined in FP64
-    T kk = (T)0, quad = (T)0, logs = (T)0, pen = (T)0, fuse = (T)0;
-    const int nt = (p + 31) / 32;
-    for (int k = blockIdx.x; k < nt * nt; k += gridDim.x) {
-      const int bi = k / nt, bj = k % nt;
-      if (bi > bj) continue;
-      // wt[m][c][r] = W_m[32 bj + r][32 bi + c]
-      for (int e = threadIdx.x; e < 2 * 1024; e += blockDim.x) {
-        const int m = e >> 10, r = (e >> 5) & 31, c = e & 31;
-        const int row = 32 * bj + r;
-        wt[m][c][r] = row < p ? __ldcg(a.W[m] + (size_t)row * ld + 32 * bi + c) : (T)0;
-      }
-      __syncthreads();
-      for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-        const int ty = e >> 5, tx = e & 31;
-        const int i = 32 * bi + ty, j = 32 * bj + tx;
-        if (i >= p || j >= p || i > j) continue;
-        const size_t ij = (size_t)i * ld + j;
-        const T x = __ldcg(a.Om[0] + ij), y = __ldcg(a.Om[1] + ij);
-        const T wa = __ldcg(a.W[0] + ij), wb = __ldcg(a.W[1] + ij);
-        if (i == j) {
-          const T ga = wa - (T)1 / x, gb = wb - (T)1 / y;
-          kk = nmax<T>(kk, diag_kkt<T>(ga, gb, x, y, l2t));
-          quad += x * wa + y * wb;
-          logs += log(x) + log(y);
-          fuse += fabs(x - y);
-        } else {
-          const T g1 = wa + wt[0][ty][tx], g2 = wb + wt[1][ty][tx];
-          kk = nmax<T>(kk, pair_kkt<T>(g1, g2, x, y, l1t, l2t));
-          quad += x * g1 + y * g2;
-          pen += fabs(x) + fabs(y);
-          fuse += fabs(x - y);
-        }
-      }
-      __syncthreads();
-    }
-    // block reduction of the partials
-    {
-      double v[kJParts] = {(double)kk, (double)quad, (double)logs, (double)pen, (double)fuse,
-                           (double)dmax, tiled ? 0.5 * (double)moved : (double)moved, 0.0};
-#pragma unroll
-      for (int q = 0; q < kJParts; ++q) {
-        double x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double y = __shfl_down_sync(kFull, x, o);
-          x = (q == kJPartKkt || q == kJPartDelta) ? nmax<double>(x, y) : x + y;
-        }
-        if (lane == 0) red[wid][q] = x;
-      }
-      __syncthreads();
-      if (threadIdx.x < kJParts) {
-        const int q = threadIdx.x;
-        double x = red[0][q];
-        for (int w = 1; w < kJointWarps; ++w)
-          x = (q == kJPartKkt || q == kJPartDelta) ? nmax<double>(x, red[w][q]) : x + red[w][q];
-        a.partials[((size_t)(evals & 1) * gridDim.x + blockIdx.x) * kJParts + q] = x;
-      }
-    }
+    JointSums<T> js;
+    joint_pass<T>(p, ld, {a.W[0], a.W[1]}, {a.Om[0], a.Om[1]}, l1t, l2t, (int)blockIdx.x,
+                  (int)gridDim.x, wt, js);
+    joint_reduce({(double)js.kk, (double)js.quad, (double)js.logs, (double)js.pen, (double)js.fuse,
+                  (double)dmax, (double)moved, 0.0},
+                 red, a.partials + ((size_t)(evals & 1) * gridDim.x + blockIdx.x) * kJParts);
     grid_barrier(a.barrier, gen, a.wait, P + 1);
     // every CTA combines the partials in the same order: the same decision
     if (wid == 0) {
@@ -605,6 +563,231 @@ __global__ void __launch_bounds__(kJointThreads, 1) k_joint(const JointArgs<T> a
   }
 }
 
+// ---- the wave form (wave.cuh): a launch per sweep and one per evaluation,
+// the iteration's state in device memory between them; launches past the end
+// return at once.
+
+struct JointState {
+  double best;
+  int t, first_delta, since_best;
+  int status;       // -1: running
+  unsigned ticket;  // CTAs of an evaluation that are through
+};
+
+struct WaveJoint {
+  float l1, l2;
+  float dmax = 0.f;
+  int moved = 0;  // both owners count a pair
+  __device__ static void denominators(const float (&c)[2], float (&dn)[3]) {
+    dn[0] = c[0];
+    dn[1] = c[1];
+    dn[2] = c[0] + c[1];
+  }
+  __device__ void pair(const float (&c)[2], const float (&rc)[3], const float (&om)[2],
+                       const float (&wa)[2], const float (&wb)[2], float (&n)[2], float (&dn)[2],
+                       float (&y)[2]) {
+    const float g1 = (wa[0] + wb[0]) - c[0] * om[0];
+    const float g2 = (wa[1] + wb[1]) - c[1] * om[1];
+    // block_pair, with the case's numerators and denominators selected
+    const float na = jsoft<float>(-(g1 + l2), l1), nb = jsoft<float>(-(g2 - l2), l1);
+    const float nc = jsoft<float>(-(g1 - l2), l1), nd = jsoft<float>(-(g2 + l2), l1);
+    const float nt = jsoft<float>(-(g1 + g2), 2.f * l1);
+    const bool first = na * c[1] > nb * c[0], second = nc * c[1] < nd * c[0];
+    n[0] = first ? na : (second ? nc : nt);
+    n[1] = first ? nb : (second ? nd : nt);
+    dn[0] = first || second ? c[0] : c[0] + c[1];
+    dn[1] = first || second ? c[1] : c[0] + c[1];
+    y[0] = first || second ? rc[0] : rc[2];
+    y[1] = first || second ? rc[1] : rc[2];
+  }
+  __device__ void count(const float (&d)[2]) {
+    dmax = nmax<float>(dmax, nmax<float>(fabsf(d[0]), fabsf(d[1])));
+    if (d[0] != 0.f || d[1] != 0.f) ++moved;
+  }
+  __device__ void diag(const WaveArgs<2>& a, int i, const float (&w)[2], float (&dd)[2]) {
+    const size_t ii = (size_t)i * a.ld + i;
+    const float o1 = a.Om[0][ii], o2 = a.Om[1][ii];
+    const float s1 = __ldg(a.S[0] + ii), s2 = __ldg(a.S[1] + ii);
+    const float b1 = w[0] - o1 * s1;
+    const float b2 = w[1] - o2 * s2;
+    float n1, n2;
+    block_diag<float>(s1, b1, s2, b2, l2, n1, n2);
+    dd[0] = n1 - o1;
+    dd[1] = n2 - o2;
+    if (dd[0] != 0.f) a.Om[0][ii] = n1;
+    if (dd[1] != 0.f) a.Om[1][ii] = n2;
+    dmax = nmax<float>(dmax, nmax<float>(fabsf(dd[0]), fabsf(dd[1])));
+  }
+};
+
+// first: the iteration starts here (the state is not set yet).
+__global__ void __launch_bounds__(kWaveThreads, 1) k_joint_wave(const __grid_constant__ JointArgs<float> a,
+                                                                int first, int cl) {
+  WaveSmem<2>& s = wave_smem<2>();
+  const JointState* st = wave_state<JointState>(a.words, a.p, 2);
+  if (!first && st->status >= 0) return;
+  if (threadIdx.x == 0) {
+    s.args.p = a.p;
+    s.args.P = a.P;
+    s.args.ld = a.ld;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      s.args.S[m] = a.S[m];
+      s.args.W[m] = a.W[m];
+      s.args.Om[m] = a.Om[m];
+      s.args.sdiag[m] = a.S[m];
+    }
+    s.args.sd_stride = (size_t)a.ld + 1;
+    s.args.words = a.words;
+    s.args.tag = a.tag + (first ? 0u : (unsigned)st->t);
+    s.args.wait = a.wait;
+  }
+  __syncthreads();
+  WaveJoint ops{(float)a.lambda1, (float)a.lambda2};
+  const int block = (int)blockIdx.x / cl, rank = (int)blockIdx.x % cl;
+  cl = wave_cluster_size(cl);
+  if (rank >= cl) return;
+  wave_sweep<2>(block, rank, cl, ops);
+  if (rank > 0) return;
+  wave_put_parts((double)ops.dmax, (double)ops.moved,
+                 wave_sweep_parts(a.words, a.p, 2) + (size_t)kWaveSweepParts * block);
+}
+
+// The evaluation (swept: after a sweep, else of the starting point); the last
+// CTA through decides.
+__global__ void __launch_bounds__(kJointThreads) k_joint_eval(const __grid_constant__ JointArgs<float> a,
+                                                              int first, int swept) {
+  __shared__ float wt[2][32][33];
+  __shared__ double red[kJointWarps][kJParts];
+  __shared__ int s_last;
+  JointState* st = wave_state<JointState>(a.words, a.p, 2);
+  if (!first && st->status >= 0) return;
+  const int G = gridDim.x;
+  double* parts = wave_eval_parts(a.words, a.p, 2);
+  JointSums<float> js;
+  joint_pass<float>(a.p, a.ld, {a.W[0], a.W[1]}, {a.Om[0], a.Om[1]}, (float)a.lambda1, (float)a.lambda2,
+                    (int)blockIdx.x, G, wt, js);
+  joint_reduce({(double)js.kk, (double)js.quad, (double)js.logs, (double)js.pen, (double)js.fuse, 0.0,
+                0.0, 0.0},
+               red, parts + (size_t)blockIdx.x * kJParts);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(&st->ticket, 1u) == (unsigned)G - 1u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  // the partials in a fixed order: lane by lane, then a tree
+  const int lane = threadIdx.x;
+  const double* sp = wave_sweep_parts(a.words, a.p, 2);
+  double x[kJParts];
+#pragma unroll
+  for (int q = 0; q < kJParts; ++q) x[q] = 0.0;
+  for (int b = lane; b < G; b += 32)
+#pragma unroll
+    for (int q = 0; q < kJParts; ++q) {
+      const double y = __ldcg(parts + (size_t)b * kJParts + q);
+      x[q] = q == kJPartKkt ? nmax<double>(x[q], y) : x[q] + y;
+    }
+  if (swept)
+    for (int b = lane; b < wave_blocks(a.p); b += 32) {
+      x[kJPartDelta] = nmax<double>(x[kJPartDelta], __ldcg(sp + (size_t)kWaveSweepParts * b));
+      x[kJPartMoved] += 0.5 * __ldcg(sp + (size_t)kWaveSweepParts * b + 1);
+    }
+#pragma unroll
+  for (int q = 0; q < kJParts; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_xor_sync(kFull, x[q], o);
+      x[q] = q == kJPartKkt || q == kJPartDelta ? nmax<double>(x[q], y) : x[q] + y;
+    }
+  if (lane != 0) return;
+  JointState w = *st;
+  if (first) {
+    w.best = INFINITY;
+    w.t = w.first_delta = w.since_best = 0;
+  }
+  w.status = -1;
+  w.ticket = 0;
+  const double kkt = x[kJPartKkt], delta = x[kJPartDelta], moved = x[kJPartMoved];
+  const double obj =
+      -x[kJPartLog] + 0.5 * x[kJPartQuad] + a.lambda1 * x[kJPartPen] + a.lambda2 * x[kJPartFuse];
+  if (swept) {
+    if (w.t < a.hist_len) {
+      double* h = a.hist + (size_t)w.t * kJHist;
+      h[0] = delta;
+      h[1] = kkt;
+      h[2] = obj;
+      h[3] = moved;
+    }
+    ++w.t;
+    if (!w.first_delta && delta < a.delta_tol) w.first_delta = w.t;
+    if (kkt < 0.9 * w.best) {
+      w.best = kkt;
+      w.since_best = 0;
+    } else {
+      ++w.since_best;
+    }
+  }
+  if (ld_relaxed_s32(a.wait.abort) != 0)
+    w.status = kJStatusAborted;
+  else if (!isfinite(kkt) || !isfinite(obj))
+    w.status = kJStatusNonfinite;
+  else if (kkt <= a.tol)
+    w.status = kJStatusConverged;
+  else if (swept && a.stall_stop && w.since_best >= kJStallSweeps)
+    w.status = kJStatusStalled;
+  else if (w.t >= a.n_sweeps)
+    w.status = kJStatusMaxSweeps;
+  *st = w;
+  if (w.status >= 0) {
+    a.result[kJResSweeps] = w.t;
+    a.result[kJResKkt] = kkt;
+    a.result[kJResObj] = obj;
+    a.result[kJResDelta] = delta;
+    a.result[kJResMoved] = moved;
+    a.result[kJResStatus] = w.status;
+    a.result[kJResFirstDelta] = w.first_delta;
+  }
+}
+
+static_assert(kWaveEvalParts == kJParts, "the evaluation's partials");
+constexpr int kWaveChunk = 4;  // sweeps between two looks at the outcome
+
+cudaError_t run_joint_wave(const JointArgs<float>& a, int grid, cudaStream_t st) {
+  const size_t dyn = sizeof(WaveSmem<2>);
+  cudaError_t e = cudaFuncSetAttribute((const void*)k_joint_wave,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  const int nb = wave_blocks(a.p), tiles = nb * nb;
+  const int G = std::max(1, std::min({tiles, 2 * grid, kWaveEvalCtas}));
+  int first = 1, status = -1, cl = 1;
+  e = wave_cluster((const void*)k_joint_wave, nb, 2, a.p, dyn, &cl);
+  if (e != cudaSuccess) return e;
+  if (a.eval_first || a.n_sweeps == 0) {
+    note_launches(1);
+    k_joint_eval<<<G, kJointThreads, 0, st>>>(a, 1, 0);
+    first = 0;
+  }
+  const int* where = &wave_state<JointState>(a.words, a.p, 2)->status;
+  for (int t = 0; status < 0; t += kWaveChunk) {
+    if (t >= a.n_sweeps + kWaveChunk) return cudaErrorUnknown;
+    for (int k = 0; k < kWaveChunk && t + k < a.n_sweeps; ++k) {
+      note_launches(2);
+      e = wave_launch(k_joint_wave, nb, cl, dyn, st, a, first, cl);
+      if (e != cudaSuccess) return e;
+      k_joint_eval<<<G, kJointThreads, 0, st>>>(a, first, 1);
+      first = 0;
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, where, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // W = Om S from the nonzero entries of each row of Om: one warp per row; the
 // row's nonzeros are gathered by ballot in batches of 32 and applied to the
 // whole W row (FP64 accumulation within a batch).
@@ -644,15 +827,8 @@ cudaError_t launch_joint_t(const JointArgs<T>& a, int grid, cudaStream_t st) {
   if (a.ld % 32 != 0 || a.p < 2 || grid < 1) return cudaErrorInvalidValue;
   void* args[] = {(void*)&a};
   note_launches(1);
-  const size_t dyn = sizeof(T) == 4 && a.words != nullptr ? sizeof(WaveSmem<2>) : 0;
-  if (dyn > 0) {
-    if (grid < wave_blocks(a.p)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_joint<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-  }
   return cudaLaunchCooperativeKernel((const void*)k_joint<T>, dim3(grid), dim3(kJointThreads),
-                                     args, dyn, st);
+                                     args, 0, st);
 }
 
 }  // namespace
@@ -661,12 +837,13 @@ cudaError_t launch_joint(const JointArgs<double>& a, int grid, cudaStream_t st) 
   return launch_joint_t(a, grid, st);
 }
 cudaError_t launch_joint(const JointArgs<float>& a, int grid, cudaStream_t st) {
-  return launch_joint_t(a, grid, st);
+  if (a.words == nullptr) return launch_joint_t(a, grid, st);
+  if (a.ld % 32 != 0 || a.p < 2 || grid < wave_blocks(a.p)) return cudaErrorInvalidValue;
+  return run_joint_wave(a, grid, st);
 }
 
 int joint_wave_blocks(int p) { return wave_blocks(p); }
-size_t joint_wave_words(int p) { return wave_words(p, 2); }
-static_assert(kWaveThreads == kJointThreads, "the wave form runs in the joint kernel's CTAs");
+size_t joint_wave_words(int p) { return wave_scratch_words(p, 2); }
 
 cudaError_t joint_occupancy(bool f32, int* blocks_per_sm) {
   return f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_joint<float>,

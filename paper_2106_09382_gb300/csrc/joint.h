@@ -57,7 +57,8 @@ struct JointArgs {
 };
 
 // One persistent cooperative launch (grid CTAs of kJointThreads threads,
-// co-resident): joint sweeps until the stopping rule or n_sweeps.
+// co-resident): joint sweeps until the stopping rule or n_sweeps.  With
+// a.words a launch per sweep and evaluation instead, and waits on the stream.
 cudaError_t launch_joint(const JointArgs<double>& a, int grid, cudaStream_t st);
 cudaError_t launch_joint(const JointArgs<float>& a, int grid, cudaStream_t st);
 // With a.words the grid has at least joint_wave_blocks(p) CTAs.

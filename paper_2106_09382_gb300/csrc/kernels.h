@@ -96,7 +96,6 @@ struct SweepArgs {
   unsigned poll_ns;          // back-off between mailbox polls (0: none)
   unsigned tag_base;
   int fault_vertex, fault_step;
-  unsigned long long* words;  // wave form: exchange words (wave.cuh); tags from tag_base
   // batched launch (launch_sweep_batch): problems and the lambda path every
   // problem walks (warm-started, n_sweeps sweeps at most per lambda)
   const BatchProblem<T>* probs;
@@ -122,14 +121,31 @@ cudaError_t sweep_occupancy(bool mixed, int block, int* blocks_per_sm);
 cudaError_t launch_sweep_batch(const SweepArgs<double>& a, int grid, int block, cudaStream_t st);
 cudaError_t launch_sweep_batch(const SweepArgs<float>& a, int grid, int block, cudaStream_t st);
 // The wave form (FP32, wave.cuh): tiles of 32 x 32 vertices instead of colour
-// steps, one CTA per block of 32 rows; the same iterates.  launch_sweep_wave:
-// grid >= wave_blocks(p) CTAs (the others join the KKT pass).  _batch: as
-// launch_sweep_batch, wave_blocks(p) CTAs per problem.
+// steps, one CTA per block of 32 rows; the same iterates.
 constexpr int kWaveMaxBlocks = 64;  // the exchange words grow with the square (35 MB here)
-cudaError_t launch_sweep_wave(const SweepArgs<float>& a, int grid, cudaStream_t st);
-cudaError_t launch_sweep_wave_batch(const SweepArgs<float>& a, int grid, cudaStream_t st);
+struct WaveLaunch {
+  BatchProblem<float> one;           // the problem (n_probs = 0), or
+  const BatchProblem<float>* probs;  // n_probs problems, wave blocks of CTAs each
+  int n_probs;
+  const double* lambdas;             // lambdas[k0 + k]; nullptr: `lambda`
+  double lambda, tol, delta_tol;
+  int stop_rule, n_sweeps, stall_stop;
+  unsigned tag0;                     // larger than any tag in the words
+  WaitCtl wait;
+  double* hist;                      // hist_len x kHist (one problem)
+  int hist_len;
+  unsigned long long* words0;        // of the first problem, and its dimension
+  int p0;
+  int eval_ctas, first, cl;          // (set by run_sweep_wave; cl: CTAs per block)
+};
+// Sweeps until every problem has met its stopping rule at every lambda it
+// walks (as launch_sweep_batch); waits on the stream.  grid: the problems'
+// blocks together, co-resident; p_max: the largest dimension; count: some
+// problem has a cnt.
+constexpr int kWaveChunk = 4;  // sweeps between two looks at the outcome
+cudaError_t run_sweep_wave(WaveLaunch a, int p_max, int grid, int sms, bool count, cudaStream_t st);
 int sweep_wave_blocks(int p);
-size_t sweep_wave_words(int p, int matrices);
+size_t sweep_wave_words(int p, int matrices);  // 64-bit words; zeroed at first
 // Largest launchable cluster (power of two <= 16; 0 if none).
 cudaError_t sweep_cluster_size(bool mixed, int block, int row_warps, int rows_per_warp, int* cs);
 

@@ -21,32 +21,9 @@
 //     KKT / objective pass; a second one publishes its partial results.
 #include "common.cuh"
 #include "kernels.h"
-#include "wave.cuh"
+#include "sweep_eval.cuh"
 
 namespace concord {
-
-template <typename T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-  using V = float4;
-  static constexpr int N = 4;
-  __device__ static void fma(V& w, float d, const V& s) {
-    w.x = fmaf(d, s.x, w.x);
-    w.y = fmaf(d, s.y, w.y);
-    w.z = fmaf(d, s.z, w.z);
-    w.w = fmaf(d, s.w, w.w);
-  }
-};
-template <>
-struct Vec16<double> {
-  using V = double2;
-  static constexpr int N = 2;
-  __device__ static void fma(V& w, double d, const V& s) {
-    w.x = ::fma(d, s.x, w.x);
-    w.y = ::fma(d, s.y, w.y);
-  }
-};
 
 __device__ __forceinline__ float fma_t(float d, float s, float w) { return fmaf(d, s, w); }
 __device__ __forceinline__ double fma_t(double d, double s, double w) { return ::fma(d, s, w); }
@@ -81,39 +58,6 @@ __device__ __forceinline__ void axpy_row(T* __restrict__ w, const T* __restrict_
     VT::fma(w0, d, s0);
     wv[k] = w0;
   }
-}
-
-template <typename T>
-__device__ __forceinline__ T soft_threshold(T x, T tau) {
-  T a = fabs(x) - tau;
-  if (!(a > (T)0)) return (T)0;
-  return x > (T)0 ? a : -a;
-}
-
-// Block reduction of the per-thread partials into partials[blockIdx.x*kParts+k].
-__device__ __forceinline__ void block_reduce_parts(double (&v)[kParts], double* out,
-                                                   double (*red)[kParts], int slot) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kParts; ++k) {
-    double x = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      double y = __shfl_down_sync(0xffffffffu, x, o);
-      x = (k == kPartKkt || k == kPartDelta) ? fmax(x, y) : x + y;
-    }
-    if (lane == 0) red[wid][k] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < kParts; ++k) {
-      double x = red[0][k];
-      for (int w = 1; w < nw; ++w)
-        x = (k == kPartKkt || k == kPartDelta) ? fmax(x, red[w][k]) : x + red[w][k];
-      out[(size_t)slot * kParts + k] = x;
-    }
-  }
-  __syncthreads();
 }
 
 // Partner of row v at the colour whose ring index is r (rows v >= 1): the
@@ -224,8 +168,6 @@ __device__ __forceinline__ bool box_read<double>(const unsigned long long* local
 //     word a row reads lives in its own CTA's shared memory and the partner
 //     stores into it through distributed shared memory (lower latency), with
 //     per-row progress counters guarding slot reuse.
-//   WAVE = true (FP32): a sweep runs tile by tile (wave.cuh) on the first
-//     wave_blocks(p) CTAs of the group; the others join the KKT pass.
 //   BATCH = true (grid form): the launch serves a.n_probs independent
 //     problems; each CTA belongs to one problem (its CTA range), whose rows,
 //     mailbox ring, barriers and partial sums are its own, and each problem
@@ -237,38 +179,7 @@ __device__ __forceinline__ const SweepArgs<T>& pick_args(const SweepArgs<T>& bat
   return use_batch ? batch : single;
 }
 
-// A sweep's pairs and diagonal in the wave form.
-struct WaveSingle {
-  const SweepArgs<float>& A;
-  float lam;
-  float dpair = 0.f;   // largest change of a pair
-  double ddiag = 0.0;  // of a diagonal entry
-  int active = 0;
-  __device__ void pair(const float (&c)[1], const float (&om)[1], const float (&wa)[1],
-                       const float (&wb)[1], float (&nw)[1]) {
-    const float x = (c[0] * om[0] - wa[0]) - wb[0];
-    const float sx = soft_threshold(x, lam);
-    nw[0] = 0.f;
-    if (sx != 0.f) nw[0] = sx / c[0];
-  }
-  __device__ void count(const float (&d)[1]) {
-    if (d[0] != 0.f) {
-      dpair = fmaxf(dpair, fabsf(d[0]));
-      ++active;
-    }
-  }
-  __device__ void diag(int i, const float (&w)[1], float (&dd)[1]) {
-    const double sii = A.sdiag64[i], oii = A.omdiag64[i];
-    const double ci = (double)w[0] - oii * sii;
-    const double nw = (-ci + sqrt(ci * ci + 4.0 * sii)) / (2.0 * sii);
-    A.omdiag64[i] = nw;
-    A.Om[(size_t)i * A.ld + i] = (float)nw;
-    dd[0] = (float)(nw - oii);
-    ddiag = fmax(ddiag, fabs(nw - oii));
-  }
-};
-
-template <typename T, bool MIXED, bool CLUSTER, bool BATCH, bool WAVE = false>
+template <typename T, bool MIXED, bool CLUSTER, bool BATCH>
 __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a) {
   using MB = Mailbox<T>;
   constexpr unsigned FULL = 0xffffffffu;
@@ -303,7 +214,6 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
       s_args.sdiag64 = q.sdiag64;
       s_args.omdiag64 = q.omdiag64;
       s_args.mbox = q.mbox;
-      s_args.words = q.words;
       s_args.barrier = q.barrier;
       s_args.partials = q.partials;
       s_args.result = q.result;
@@ -324,7 +234,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
     cta = s_gc[1];
   }
   const SweepArgs<T>& A = pick_args<T>(s_args, a, BATCH);
-  const bool row_warp = WAVE || wid < A.row_warps;
+  const bool row_warp = wid < A.row_warps;
   const int p = A.p, P = A.P, ld = A.ld;
   const int pe = P + 1;
   const int R = A.rows_per_warp;
@@ -335,12 +245,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
   int myrow;
   if constexpr (CLUSTER) {
     myrow = li * CS + (int)cta;
-  } else if constexpr (WAVE) {
-    myrow = lane < 2 ? cta * kWaveB + 2 * wid + lane : A.p;
   } else {
     myrow = (cta * A.row_warps + wid) + lane * (G * A.row_warps);
   }
-  const bool has_row = row_warp && (WAVE || lane < R) && myrow < p;
+  const bool has_row = row_warp && lane < R && myrow < p;
   // the lambda in force (batch: walks the path, index kl)
   double lam_cur = A.lambda;
   T lam = (T)lam_cur;
@@ -385,26 +293,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
   for (;;) {
     const bool do_sweep = !A.kkt_only && (BATCH ? t_lam : t) < A.n_sweeps;
     double dmax = 0.0, nact = 0.0;
-    if constexpr (WAVE) {
-      if (do_sweep && cta < wave_blocks(p)) {
-        WaveArgs<1> wa;
-        wa.p = p;
-        wa.P = P;
-        wa.ld = ld;
-        wa.S[0] = A.S;
-        wa.W[0] = A.W;
-        wa.Om[0] = A.Om;
-        wa.sdiag[0] = A.sdiag;
-        wa.sd_stride = 1;
-        wa.words = A.words;
-        wa.tag = A.tag_base + (unsigned)t;
-        wa.wait = wc;
-        WaveSingle ops{A, lam};
-        wave_sweep<1>(wa, *reinterpret_cast<WaveSmem<1>*>(dyn), cta, ops);
-        dmax = fmax((double)ops.dpair, ops.ddiag);
-        nact = (double)ops.active;
-      }
-    } else if (do_sweep && row_warp) {
+    if (do_sweep && row_warp) {
       const unsigned step0 = tag_base + (unsigned)(t * P);
       int cnt = 0;  // pending updates of this lane's row
       // Partners without integer division: for v >= 1 the ring index
@@ -726,94 +615,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
     for (int k = 0; k < kParts; ++k) v[k] = 0.0;
     v[kPartDelta] = dmax;
     v[kPartActive] = nact;
-    {
-      // Work unit: an 8-row chunk of a 32 x 32 tile (ta <= tb) of the upper
-      // triangle.  Lane l takes column j = tb*32 + l: W_ij comes from row i
-      // (coalesced across lanes), W_ji from row j as one 8-element vector, so
-      // G_ij = W_ij + W_ji pairs up without a transpose.
-      using VT = Vec16<T>;
-      using V = typename VT::V;
-      constexpr int NV = 8 / VT::N;
-      const int nb = (p + kTile - 1) / kTile;
-      const double lamd = lam_cur;
-      const float lamf = (float)lam_cur;
-      const int units = nb * nb * 4;
-      const int gwarps = G * (blockDim.x >> 5);
-      for (int u = cta * (blockDim.x >> 5) + wid; u < units; u += gwarps) {
-        const int tau = u >> 2, r0 = (u & 3) * 8;
-        const int ta = tau / nb, tb = tau % nb;
-        if (ta > tb) continue;
-        const int j = tb * kTile + lane;
-        const int i0 = ta * kTile + r0;
-        if (i0 >= p) continue;
-        T w1[8], om8[8], wt[8];
-        const bool jv = j < p;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int i = i0 + r;
-          const bool ok = jv && i < p;
-          w1[r] = ok ? __ldcg(A.W + (size_t)i * ld + j) : (T)0;
-          om8[r] = ok ? __ldcg(A.Om + (size_t)i * ld + j) : (T)0;
-        }
-        if (jv) {
-          const V* src = reinterpret_cast<const V*>(A.W + (size_t)j * ld + i0);
-#pragma unroll
-          for (int q = 0; q < NV; ++q) {
-            V x = __ldcg(src + q);
-            if constexpr (VT::N == 4) {
-              wt[4 * q + 0] = ((const float*)&x)[0];
-              wt[4 * q + 1] = ((const float*)&x)[1];
-              wt[4 * q + 2] = ((const float*)&x)[2];
-              wt[4 * q + 3] = ((const float*)&x)[3];
-            } else {
-              wt[2 * q + 0] = ((const double*)&x)[0];
-              wt[2 * q + 1] = ((const double*)&x)[1];
-            }
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) wt[r] = (T)0;
-        }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int i = i0 + r;
-          if (!jv || i >= p) continue;
-          if (i < j) {
-            const T om_t = om8[r];
-            // FP32 screen: a zero entry whose |G_ij| is clearly below lambda
-            // has residual exactly 0 (the margin covers the FP32 rounding of
-            // G); every other entry is evaluated in FP64.
-            const float w1f = (float)w1[r], w2f = (float)wt[r];
-            const float gf = w1f + w2f;
-            if (om_t == (T)0 && fabsf(gf) <= lamf - 1e-5f * (1.0f + fabsf(w1f) + fabsf(w2f)))
-              continue;
-            const double om = (double)om_t;
-            const double g = (double)w1[r] + (double)wt[r];
-            double res;
-            if (om > 0.0)
-              res = fabs(g + lamd);
-            else if (om < 0.0)
-              res = fabs(g - lamd);
-            else
-              res = fmax(fabs(g) - lamd, 0.0);
-            v[kPartKkt] = fmax(v[kPartKkt], res);
-            v[kPartQuad] += om * g;
-            v[kPartPen] += fabs(om);
-            if (!isfinite(g) || !isfinite(om)) v[kPartBad] += 1.0;
-          } else if (i == j) {
-            const double wii = (double)w1[r];
-            const double oii = MIXED ? __ldcg(A.omdiag64 + i) : (double)om8[r];
-            if (oii > 0.0 && isfinite(wii) && isfinite(oii)) {
-              v[kPartKkt] = fmax(v[kPartKkt], fabs(wii - 1.0 / oii));
-              v[kPartQuad] += oii * wii;
-              v[kPartLog] += log(oii);
-            } else {
-              v[kPartBad] += 1.0;
-            }
-          }
-        }
-      }
-    }
+    kkt_pass<T, MIXED>(p, ld, A.W, A.Om, A.omdiag64, lam_cur, cta, G, v);
     block_reduce_parts(v, A.partials, red, cta);
     if constexpr (CLUSTER)
       cluster_sync_all();
@@ -903,11 +705,9 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(const SweepArgs<T> a
             const int i = __shfl_sync(FULL, myrow, k);
             const T* orow = A.Om + (size_t)i * ld;
             for (int x = lane; x < p; x += 32)
-              if (__ldcg(orow + x) != (T)0) atomicAdd(cnt_k + (size_t)i * p + x, 1.0f);
+              if (orow[x] != (T)0) atomicAdd(cnt_k + (size_t)i * p + x, 1.0f);
           }
         }
-        // (wave form: row 0 is written by every CTA of the group)
-        if (WAVE && A.batch_cnt && s_lam_count) group_barrier(A.barrier, gen, G, wc, 3000000 + t, cta);
         if (!s_stop) {
           ++kl;
           lam_cur = A.lambdas[kl];
@@ -1025,28 +825,6 @@ cudaError_t launch_sweep_batch(const SweepArgs<double>& a, int grid, int block, 
 cudaError_t launch_sweep_batch(const SweepArgs<float>& a, int grid, int block, cudaStream_t st) {
   return launch_sweep_batch_impl<float, true>(a, grid, block, st);
 }
-
-cudaError_t launch_sweep_wave(const SweepArgs<float>& args, int grid, cudaStream_t st) {
-  const size_t dyn = sizeof(WaveSmem<1>);
-  const void* fn = (const void*)k_sweep<float, true, false, false, true>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  if (e != cudaSuccess) return e;
-  note_launches(1);
-  void* kargs[] = {(void*)&args};
-  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveThreads), kargs, dyn, st);
-}
-cudaError_t launch_sweep_wave_batch(const SweepArgs<float>& args, int grid, cudaStream_t st) {
-  const size_t dyn = sizeof(WaveSmem<1>);
-  const void* fn = (const void*)k_sweep<float, true, false, true, true>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  if (e != cudaSuccess) return e;
-  note_launches(1);
-  void* kargs[] = {(void*)&args};
-  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kWaveThreads), kargs, dyn, st);
-}
-int sweep_wave_blocks(int p) { return wave_blocks(p); }
-size_t sweep_wave_words(int p, int matrices) { return wave_words(p, matrices); }
-static_assert(kWaveThreads == kSweepThreads, "the wave form runs in the sweep kernel's CTAs");
 
 cudaError_t sweep_occupancy(bool mixed, int block, int* blocks_per_sm) {
   return mixed ? sweep_occupancy_impl<float, true>(block, blocks_per_sm)

@@ -1,0 +1,281 @@
+// Sweeps in the wave form (wave.cuh) for a single problem or several: pairs of
+// launches, a sweep and its evaluation, that hand the iteration's state on in
+// device memory; launches past the end of every problem return at once, so
+// the host looks at the outcome once in a few sweeps only.  (A persistent
+// kernel over the sweeps spills registers in the colour steps, whatever is
+// kept from sweep to sweep in shared memory, and evaluates on the sweep's
+// CTAs alone.)
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+#include "sweep_eval.cuh"
+#include "wave.cuh"
+
+namespace concord {
+namespace {
+
+struct WaveState {
+  double best;         // smallest KKT residual at this lambda
+  int t, t_lam;        // sweeps so far, at this lambda
+  int kl;              // lambda
+  int first_delta, since_best;
+  int done;
+  int count;           // lambda whose support is to be counted (-1: none)
+  int remaining;       // (first problem) problems that are not done
+  unsigned ticket;     // CTAs of an evaluation that are through
+};
+
+// A sweep's pairs and diagonal.
+struct WaveSingle {
+  const double* sdiag64;
+  double* omdiag64;
+  float lam;
+  float dpair = 0.f;   // largest change of a pair
+  double ddiag = 0.0;  // of a diagonal entry
+  int active = 0;      // both owners count a pair
+  __device__ static void denominators(const float (&c)[1], float (&dn)[1]) { dn[0] = c[0]; }
+  __device__ void pair(const float (&c)[1], const float (&rc)[1], const float (&om)[1],
+                       const float (&wa)[1], const float (&wb)[1], float (&n)[1], float (&dn)[1],
+                       float (&y)[1]) {
+    n[0] = soft_threshold((c[0] * om[0] - wa[0]) - wb[0], lam);
+    dn[0] = c[0];
+    y[0] = rc[0];
+  }
+  __device__ void count(const float (&d)[1]) {
+    dpair = fmaxf(dpair, fabsf(d[0]));
+    active += d[0] != 0.f ? 1 : 0;
+  }
+  __device__ void diag(const WaveArgs<1>& a, int i, const float (&w)[1], float (&dd)[1]) {
+    const double sii = sdiag64[i], oii = omdiag64[i];
+    const double ci = (double)w[0] - oii * sii;
+    const double nw = (-ci + sqrt(ci * ci + 4.0 * sii)) / (2.0 * sii);
+    omdiag64[i] = nw;
+    a.Om[0][(size_t)i * a.ld + i] = (float)nw;
+    dd[0] = (float)(nw - oii);
+    ddiag = fmax(ddiag, fabs(nw - oii));
+  }
+};
+
+__device__ __forceinline__ double lambda_at(const WaveLaunch& a, const BatchProblem<float>& q, int kl) {
+  return a.lambdas ? a.lambdas[q.k0 + kl] : a.lambda;
+}
+
+__global__ void __launch_bounds__(kWaveThreads, 1) k_wave(const __grid_constant__ WaveLaunch a) {
+  WaveSmem<1>& s = wave_smem<1>();
+  __shared__ struct {
+    const double* sdiag64;
+    double *omdiag64, *parts;
+    float lam;
+    int block, done;
+  } g;
+  if (threadIdx.x == 0) {
+    const BatchProblem<float>* q = &a.one;
+    if (a.n_probs > 0) {
+      int lo = 0, hi = a.n_probs - 1;
+      while (lo < hi) {  // last problem whose range starts at or before this CTA
+        const int mid = (lo + hi + 1) >> 1;
+        if (a.probs[mid].cta0 <= (int)blockIdx.x / a.cl) lo = mid; else hi = mid - 1;
+      }
+      q = a.probs + lo;
+    }
+    const WaveState* st = wave_state<WaveState>(q->words, q->p, 1);
+    if (a.first && blockIdx.x == 0)
+      wave_state<WaveState>(q->words, q->p, 1)->remaining = a.n_probs > 0 ? a.n_probs : 1;
+    g.done = a.first ? 0 : st->done;
+    g.lam = (float)lambda_at(a, *q, a.first || g.done ? 0 : st->kl);
+    g.block = (int)blockIdx.x / a.cl - q->cta0;
+    g.sdiag64 = q->sdiag64;
+    g.omdiag64 = q->omdiag64;
+    g.parts = wave_sweep_parts(q->words, q->p, 1) + (size_t)kWaveSweepParts * g.block;
+    s.args.p = q->p;
+    s.args.P = q->P;
+    s.args.ld = q->ld;
+    s.args.S[0] = q->S;
+    s.args.W[0] = q->W;
+    s.args.Om[0] = q->Om;
+    s.args.sdiag[0] = q->sdiag;
+    s.args.sd_stride = 1;
+    s.args.words = q->words;
+    s.args.tag = a.tag0 + (a.first ? 0u : (unsigned)st->t);
+    s.args.wait = a.wait;
+  }
+  __syncthreads();
+  if (g.done) return;
+  WaveSingle ops{g.sdiag64, g.omdiag64, g.lam};
+  const int rank = (int)blockIdx.x % a.cl, cl = wave_cluster_size(a.cl);
+  if (rank >= cl) return;
+  wave_sweep<1>(g.block, rank, cl, ops);
+  if (rank > 0) return;
+  wave_put_parts(fmax((double)ops.dpair, ops.ddiag), (double)ops.active, g.parts);
+}
+
+// The evaluation after a sweep, a.eval_ctas CTAs per problem; the last one
+// through decides.
+__global__ void __launch_bounds__(256) k_wave_eval(const __grid_constant__ WaveLaunch a) {
+  __shared__ double red[256 / 32][kParts];
+  __shared__ int s_last;
+  const BatchProblem<float>& q = a.n_probs > 0 ? a.probs[blockIdx.x / a.eval_ctas] : a.one;
+  const int G = a.eval_ctas, cta = (int)blockIdx.x % G;
+  WaveState* st = wave_state<WaveState>(q.words, q.p, 1);
+  if (!a.first && st->done) {
+    if (cta == 0 && threadIdx.x == 0) st->count = -1;
+    return;
+  }
+  const int kl = a.first ? 0 : st->kl;
+  const double lam = lambda_at(a, q, kl);
+  double* parts = wave_eval_parts(q.words, q.p, 1);
+  double v[kParts];
+#pragma unroll
+  for (int k = 0; k < kParts; ++k) v[k] = 0.0;
+  kkt_pass<float, true>(q.p, q.ld, q.W, q.Om, q.omdiag64, lam, cta, G, v);
+  block_reduce_parts(v, parts, red, cta);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(&st->ticket, 1u) == (unsigned)G - 1u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  // the partials in a fixed order: lane by lane, then a tree
+  const int lane = threadIdx.x;
+  const double* sp = wave_sweep_parts(q.words, q.p, 1);
+  double x[kParts];
+#pragma unroll
+  for (int k = 0; k < kParts; ++k) x[k] = 0.0;
+  for (int b = lane; b < G; b += 32)
+#pragma unroll
+    for (int k = 0; k < kParts; ++k) {
+      const double y = __ldcg(parts + (size_t)b * kParts + k);
+      x[k] = k == kPartKkt ? fmax(x[k], y) : x[k] + y;
+    }
+  x[kPartDelta] = x[kPartActive] = 0.0;
+  for (int b = lane; b < wave_blocks(q.p); b += 32) {
+    x[kPartDelta] = fmax(x[kPartDelta], __ldcg(sp + (size_t)kWaveSweepParts * b));
+    x[kPartActive] += __ldcg(sp + (size_t)kWaveSweepParts * b + 1);
+  }
+#pragma unroll
+  for (int k = 0; k < kParts; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_xor_sync(0xffffffffu, x[k], o);
+      x[k] = k == kPartKkt || k == kPartDelta ? fmax(x[k], y) : x[k] + y;
+    }
+  if (lane != 0) return;
+  WaveState w = *st;
+  if (a.first) {
+    w.best = 1e300;
+    w.t = w.t_lam = w.kl = w.first_delta = w.since_best = w.done = 0;
+  }
+  w.ticket = 0;
+  w.count = -1;
+  const double kkt = x[kPartKkt], dl = x[kPartDelta], ac = x[kPartActive];
+  const double obj = -x[kPartLog] + 0.5 * x[kPartQuad] + lam * x[kPartPen];
+  const bool aborted = ld_relaxed_s32(a.wait.abort) != 0;
+  const bool nonfinite = x[kPartBad] > 0.0 || !isfinite(obj) || !isfinite(kkt);
+  const int n_sweeps = q.n_sweeps > 0 ? q.n_sweeps : a.n_sweeps;
+  const int sweeps = w.t_lam + 1;
+  if (w.first_delta == 0 && dl < a.delta_tol) w.first_delta = sweeps;
+  const bool conv = a.stop_rule == 1 ? dl < a.tol : kkt <= a.tol;
+  // stall: the KKT residual has not dropped by 10% for 4 sweeps (the FP32
+  // rounding floor)
+  bool stalled = false;
+  if (kkt < 0.9 * w.best) {
+    w.best = kkt;
+    w.since_best = 0;
+  } else if (++w.since_best >= 4 && a.stall_stop) {
+    stalled = true;
+  }
+  if (w.t < a.hist_len) {
+    double* h = a.hist + (size_t)w.t * kHist;
+    h[0] = dl;
+    h[1] = kkt;
+    h[2] = obj;
+    h[3] = ac * 0.5;
+  }
+  ++w.t;
+  ++w.t_lam;
+  if (aborted || nonfinite || conv || stalled || sweeps >= n_sweeps) {
+    double* r = q.result + (size_t)kl * kRes;
+    r[kResSweeps] = sweeps;
+    r[kResKkt] = kkt;
+    r[kResObj] = obj;
+    r[kResDelta] = dl;
+    r[kResActive] = ac * 0.5;  // each pair is counted by both owners
+    r[kResFirstDelta] = w.first_delta;
+    r[kResStatus] = aborted ? 3.0 : (nonfinite ? 2.0 : (conv ? 0.0 : (stalled ? 4.0 : 1.0)));
+    // a lambda that ends on the stall rule ends the walk when asked: the host
+    // polishes it in FP64 and counts its support then
+    const bool brk = stalled && q.stall_break;
+    if (q.cnt && !brk && !aborted) w.count = kl;
+    w.best = 1e300;
+    w.t_lam = w.first_delta = w.since_best = 0;
+    if (aborted || nonfinite || brk || kl + 1 >= q.nk)
+      w.done = 1;
+    else
+      ++w.kl;
+  }
+  const BatchProblem<float>& q0 = a.n_probs > 0 ? a.probs[0] : a.one;
+  int* remaining = &wave_state<WaveState>(q0.words, q0.p, 1)->remaining;
+  st->best = w.best;
+  st->t = w.t;
+  st->t_lam = w.t_lam;
+  st->kl = w.kl;
+  st->first_delta = w.first_delta;
+  st->since_best = w.since_best;
+  st->done = w.done;
+  st->count = w.count;
+  st->ticket = 0;
+  if (w.done) atomicSub(remaining, 1);
+}
+
+// The support of a finished lambda's solution into its slice of the counts.
+__global__ void __launch_bounds__(256) k_wave_count(const __grid_constant__ WaveLaunch a) {
+  const BatchProblem<float>& q = a.n_probs > 0 ? a.probs[blockIdx.x / a.eval_ctas] : a.one;
+  const int kl = wave_state<WaveState>(q.words, q.p, 1)->count;
+  if (kl < 0 || !q.cnt) return;
+  float* cnt = q.cnt + (size_t)kl * q.p * q.p;
+  for (int i = (int)blockIdx.x % a.eval_ctas; i < q.p; i += a.eval_ctas)
+    for (int x = threadIdx.x; x < q.p; x += blockDim.x)
+      if (q.Om[(size_t)i * q.ld + x] != 0.f) atomicAdd(cnt + (size_t)i * q.p + x, 1.0f);
+}
+
+}  // namespace
+
+int sweep_wave_blocks(int p) { return wave_blocks(p); }
+size_t sweep_wave_words(int p, int matrices) { return wave_scratch_words(p, matrices); }
+static_assert(kWaveEvalParts == kParts, "the evaluation's partials");
+
+cudaError_t run_sweep_wave(WaveLaunch a, int p_max, int grid, int sms, bool count, cudaStream_t st) {
+  const int np = std::max(a.n_probs, 1);
+  // eight units of the KKT pass per CTA (a unit per warp), two CTAs per SM at most
+  const int nb = wave_blocks(p_max), units = 2 * nb * (nb + 1);
+  a.eval_ctas = std::max(1, std::min({(units + 7) / 8, 2 * sms / np, kWaveEvalCtas}));
+  const size_t dyn = sizeof(WaveSmem<1>);
+  cudaError_t e = cudaFuncSetAttribute((const void*)k_wave, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)dyn);
+  if (e != cudaSuccess) return e;
+  e = wave_cluster((const void*)k_wave, grid, 1, p_max, dyn, &a.cl);
+  if (e != cudaSuccess) return e;
+  int left = 1;
+  a.first = 1;
+  while (left > 0) {  // (every evaluation brings a problem nearer its sweep limits)
+    for (int k = 0; k < kWaveChunk; ++k) {
+      note_launches(count ? 3 : 2);
+      e = wave_launch(k_wave, grid, a.cl, dyn, st, a);
+      if (e != cudaSuccess) return e;
+      k_wave_eval<<<np * a.eval_ctas, 256, 0, st>>>(a);
+      if (count) k_wave_count<<<np * a.eval_ctas, 256, 0, st>>>(a);
+      a.first = 0;
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&left, &wave_state<WaveState>(a.words0, a.p0, 1)->remaining, sizeof(int),
+                          cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace concord
