@@ -216,12 +216,21 @@ struct RunOut {
   int partial = 0;                  // screened sweeps that verified only their loud rows
 };
 
+// Whether the FP32 sweeps the screened kernel hands over take the wave form.
+bool dense_wave(concord_state* st) {
+  const int blocks = sweep_wave_blocks(st->p);
+  return blocks <= kWaveMaxBlocks && blocks <= st->sms && st->max_ctas == 0;
+}
+
 // One persistent launch: n_sweeps outer iterations (fewer if the stopping
 // rule holds first), or only the objective / KKT pass when kkt_only.
+// bandwidth (sweeps handed over by the screened kernel): until a sweep changes
+// fewer than active_below pairs, or one sweep.
 template <typename T>
 int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* omdiag64,
                  double lambda, double tol, int stop_rule, int n_sweeps, int kkt_only,
-                 int hist_offset, int stall_stop, RunOut* out, bool bandwidth = false) {
+                 int hist_offset, int stall_stop, RunOut* out, bool bandwidth = false,
+                 double active_below = 0.0) {
   const int p = st->p;
   const bool mixed = sizeof(T) == 4;
   // `row_warps` warps of each CTA own rows (one row per lane, up to `R` rows
@@ -238,8 +247,8 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   // bandwidth: sweeps handed over by the screened kernel change most pairs;
   // in FP32 they take the wave form (p = 1000: 3.3 ms a sweep colour by
   // colour), else the grid layout with one row per warp (all SMs stream rows)
-  const bool wave = bandwidth && mixed && !kkt_only && sweep_wave_blocks(p) <= kWaveMaxBlocks &&
-                    sweep_wave_blocks(p) <= st->sms && st->max_ctas == 0;
+  const bool wave = bandwidth && mixed && !kkt_only && dense_wave(st);
+  if (bandwidth && !wave) n_sweeps = 1;
   const int variant = bandwidth    ? CONCORD_SWEEP_GRID
                       : layout_set ? st->sweep_variant
                                    : (mixed ? CONCORD_SWEEP_CLUSTER : CONCORD_SWEEP_GRID);
@@ -375,6 +384,7 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
       w.stop_rule = stop_rule;
       w.n_sweeps = n_sweeps;
       w.stall_stop = stall_stop;
+      w.active_below = active_below;
       w.tag0 = st->wave_tag;
       w.wait = a.wait;
       w.hist = a.hist;
@@ -661,8 +671,8 @@ int launch_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* om
         return CONCORD_OK;
       }
       RunOut dq;
-      rc = launch_dense<T>(st, S, W, Om, sdiagT, omdiag64, lambda, tol, stop_rule, 1, 0,
-                           hist_offset + done, 0, &dq, true);
+      rc = launch_dense<T>(st, S, W, Om, sdiagT, omdiag64, lambda, tol, stop_rule, n_sweeps - done, 0,
+                           hist_offset + done, 0, &dq, true, 0.5 * st->nc_cap);
       if (dq.first_delta && !first_delta) first_delta = done + dq.first_delta;
       done += dq.sweeps;
       dense += dq.sweeps;

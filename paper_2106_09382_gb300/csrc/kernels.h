@@ -130,6 +130,7 @@ struct WaveLaunch {
   const double* lambdas;             // lambdas[k0 + k]; nullptr: `lambda`
   double lambda, tol, delta_tol;
   int stop_rule, n_sweeps, stall_stop;
+  double active_below;               // a sweep that changes fewer pairs is the last
   unsigned tag0;                     // larger than any tag in the words
   WaitCtl wait;
   double* hist;                      // hist_len x kHist (one problem)

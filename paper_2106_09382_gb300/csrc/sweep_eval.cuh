@@ -79,6 +79,7 @@ __device__ __forceinline__ void kkt_pass(int p, int ld, const T* W, const T* Om,
   const float lamf = (float)lam;
   const int units = nb * nb * 4;
   const int gwarps = G * (blockDim.x >> 5);
+  long long kkt = __double_as_longlong(v[kPartKkt]);
   for (int u = cta * (blockDim.x >> 5) + wid; u < units; u += gwarps) {
     const int tau = u >> 2, r0 = (u & 3) * 8;
     const int ta = tau / nb, tb = tau % nb;
@@ -117,42 +118,53 @@ __device__ __forceinline__ void kkt_pass(int p, int ld, const T* W, const T* Om,
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const int i = i0 + r;
-      if (!jv || i >= p) continue;
-      if (i < j) {
-        const T om_t = om8[r];
-        // FP32 screen: a zero entry whose |G_ij| is clearly below lambda
-        // has residual exactly 0 (the margin covers the FP32 rounding of
-        // G); every other entry is evaluated in FP64.
-        const float w1f = (float)w1[r], w2f = (float)wt[r];
-        const float gf = w1f + w2f;
-        if (om_t == (T)0 && fabsf(gf) <= lamf - 1e-5f * (1.0f + fabsf(w1f) + fabsf(w2f)))
-          continue;
-        const double om = (double)om_t;
-        const double g = (double)w1[r] + (double)wt[r];
-        double res;
-        if (om > 0.0)
-          res = fabs(g + lamd);
-        else if (om < 0.0)
-          res = fabs(g - lamd);
-        else
-          res = fmax(fabs(g) - lamd, 0.0);
-        v[kPartKkt] = fmax(v[kPartKkt], res);
-        v[kPartQuad] += om * g;
-        v[kPartPen] += fabs(om);
-        if (!isfinite(g) || !isfinite(om)) v[kPartBad] += 1.0;
-      } else if (i == j) {
-        const double wii = (double)w1[r];
-        const double oii = MIXED ? __ldcg(omdiag64 + i) : (double)om8[r];
-        if (oii > 0.0 && isfinite(wii) && isfinite(oii)) {
-          v[kPartKkt] = fmax(v[kPartKkt], fabs(wii - 1.0 / oii));
-          v[kPartQuad] += oii * wii;
-          v[kPartLog] += log(oii);
-        } else {
-          v[kPartBad] += 1.0;
+      if (!jv || i >= j) continue;
+      const T om_t = om8[r];
+      // FP32 screen: a zero entry whose |G_ij| is clearly below lambda
+      // has residual exactly 0 (the margin covers the FP32 rounding of
+      // G); every other entry is evaluated in FP64.
+      const float w1f = (float)w1[r], w2f = (float)wt[r];
+      const float gf = w1f + w2f;
+      if (om_t == (T)0 && fabsf(gf) <= lamf - 1e-5f * (1.0f + fabsf(w1f) + fabsf(w2f)))
+        continue;
+      // |G + lambda sign(om)|, or |G| - lambda where om = 0: one sum on every
+      // lane, the maximum of doubles >= 0 as integers (the FP64 pipe issues a
+      // warp over 16 cycles; three branches of it took 78 us of a sweep's
+      // evaluation at p = 1000)
+      const double g = (double)w1[r] + (double)wt[r];
+      const bool neg = __double2hiint(g) < 0;
+      const bool edge = om_t > (T)0 || om_t < (T)0;
+      const double t = g + ((edge ? om_t > (T)0 : neg) ? lamd : -lamd);
+      const bool flip = edge ? __double2hiint(t) < 0 : neg;
+      const long long res = __double_as_longlong(t) ^ (flip ? 0x8000000000000000ll : 0ll);
+      if (res > kkt && res <= 0x7ff0000000000000ll) kkt = res;  // (not a NaN)
+      if (om_t != (T)0) {
+        v[kPartQuad] += (double)om_t * g;
+        v[kPartPen] += fabs((double)om_t);
+      }
+      if (!isfinite(om_t) || (sizeof(T) == 4 ? !(isfinite(w1[r]) && isfinite(wt[r])) : !isfinite(g)))
+        v[kPartBad] += 1.0;
+    }
+    const int k = lane - r0;  // the diagonal: at most one entry per lane
+    if (ta == tb && k >= 0 && k < 8 && jv) {
+      double wii = 0.0, oii = 0.0;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r == k) {
+          wii = (double)w1[r];
+          oii = (double)om8[r];
         }
+      if (MIXED) oii = __ldcg(omdiag64 + j);
+      if (oii > 0.0 && isfinite(wii) && isfinite(oii)) {
+        kkt = max(kkt, __double_as_longlong(fabs(wii - 1.0 / oii)));
+        v[kPartQuad] += oii * wii;
+        v[kPartLog] += log(oii);
+      } else {
+        v[kPartBad] += 1.0;
       }
     }
   }
+  v[kPartKkt] = __longlong_as_double(kkt);
 }
 
 }  // namespace concord

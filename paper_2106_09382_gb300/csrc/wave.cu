@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(256) k_wave_eval(const __grid_constant__ WaveL
   }
   ++w.t;
   ++w.t_lam;
-  if (aborted || nonfinite || conv || stalled || sweeps >= n_sweeps) {
+  if (aborted || nonfinite || conv || stalled || sweeps >= n_sweeps || ac * 0.5 < a.active_below) {
     double* r = q.result + (size_t)kl * kRes;
     r[kResSweeps] = sweeps;
     r[kResKkt] = kkt;
@@ -257,10 +257,11 @@ cudaError_t run_sweep_wave(WaveLaunch a, int p_max, int grid, int sms, bool coun
   if (e != cudaSuccess) return e;
   e = wave_cluster((const void*)k_wave, grid, 1, p_max, dyn, &a.cl);
   if (e != cudaSuccess) return e;
+  const int chunk = a.n_probs > 0 ? kWaveChunk : std::min(kWaveChunk, std::max(a.n_sweeps, 1));
   int left = 1;
   a.first = 1;
   while (left > 0) {  // (every evaluation brings a problem nearer its sweep limits)
-    for (int k = 0; k < kWaveChunk; ++k) {
+    for (int k = 0; k < chunk; ++k) {
       note_launches(count ? 3 : 2);
       e = wave_launch(k_wave, grid, a.cl, dyn, st, a);
       if (e != cudaSuccess) return e;

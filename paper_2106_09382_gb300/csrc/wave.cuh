@@ -255,6 +255,12 @@ __device__ __forceinline__ void wave_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+__device__ __forceinline__ void wave_arrive(int id, int threads) {
+  __threadfence_block();
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
 // The block's CTAs meet (cl of them; every thread).
 __device__ __forceinline__ void wave_meet(int cl) {
   __syncwarp();
@@ -317,15 +323,20 @@ __device__ __forceinline__ void wave_apply(float (&y)[4], const float (*d)[16][1
 // of eight rows (row parity x half of the rows) of a matrix; of the rows of S
 // that any of the eight needs eight are requested together, the others are
 // not read.
+// signal: barrier 3 hears of the first columns as soon as they are done.
 template <int NM>
 __device__ __forceinline__ void wave_bulk(const WaveArgs<NM>& a, const WaveSmem<NM>& s, int i0, int Jb,
                                           int db, bool with0, int par, int ex0, int ex1, int w, int nw,
-                                          int nw0, int lane) {
+                                          int nw0, int lane, bool signal) {
   const int p = a.p;
   const int nv = a.ld >> 1;
   const int n0 = 4 * NM, items = n0 * ((nv + 31) >> 5);
   for (int it = w < nw0 && w < n0 ? w : n0 + w; it < items;
        it = it >= n0 ? it + nw : (it + nw0 < n0 ? it + nw0 : n0 + w)) {
+    if (signal && it >= n0) {
+      wave_arrive(3, kWaveThreads);
+      signal = false;
+    }
     const int g = it & 3, rp = g & 1, hf = g >> 1;
     const int m = NM == 1 ? 0 : (it >> 2) % NM, q = 32 * ((it >> 2) / NM) + lane;
     const unsigned need = with0 ? 0xffffu : s.need[db][m][g];
@@ -368,6 +379,7 @@ __device__ __forceinline__ void wave_bulk(const WaveArgs<NM>& a, const WaveSmem<
     for (int r = 0; r < 8; ++r)
       if (i + 2 * r >= 1 && i + 2 * r < p) Wr[2 * r * nv] = acc[r];
   }
+  if (signal) wave_arrive(3, kWaveThreads);
 }
 
 // x = lane's row of a skewed block.
@@ -708,7 +720,7 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
     if (Jp >= 0) {
       if (rank > 0) copy_changes((v - 1) & 1);
       wave_bulk<NM>(a, s, i0, Jp, (v - 1) & 1, diag0, par_p, -1, -1, kWaveWarps * rank + wid,
-                    kWaveWarps * cl, kWaveWarps, lane);
+                    kWaveWarps * cl, kWaveWarps, lane, false);
     }
     wave_meet(cl);
   };
@@ -756,7 +768,7 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
       if (Jp >= 0) {
         copy_changes((v - 1) & 1);
         wave_bulk<NM>(a, s, i0, Jp, (v - 1) & 1, diag0, par_p, t.J, nx.J,
-                      kWaveRestWarps + kWaveWarps * (rank - 1) + wid, nw, kWaveRestWarps, lane);
+                      kWaveRestWarps + kWaveWarps * (rank - 1) + wid, nw, kWaveRestWarps, lane, false);
       }
       diag0 = I == t.J && (t.hi & 1) == 0;
       par_p = t.hi & 1;
@@ -957,18 +969,18 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
       const int J = t.J, db = v & 1;
       const bool with0 = I == J && (t.hi & 1) == 0;
       if (nx.J >= 0) fetch(nx, J, wave_tile(I, nb, P, v + 2), db ^ 1, nx.J == J ? -1 : ob ^ 1);
+      if (zwarp && with0) {
+        while (zdone - 1 > I) zapply(--zdone, true);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) s.z[m][lane] = Z[m];
+      }
       if (Jp >= 0)
         wave_bulk<NM>(a, s, i0, Jp, db ^ 1, diag0, par_p, J, nx.J, wid - kWaveFirst / 32, nw,
-                      kWaveRestWarps, lane);
-      if (zwarp) {
+                      kWaveRestWarps, lane, with0);
+      else if (with0)
+        wave_arrive(3, kWaveThreads);
+      if (zwarp && !with0)
         while (zdone > 0 && zdone - 1 != I && zapply(zdone - 1, false)) --zdone;
-        if (with0) {
-          while (zdone - 1 > I) zapply(--zdone, true);
-#pragma unroll
-          for (int m = 0; m < NM; ++m) s.z[m][lane] = Z[m];
-        }
-      }
-      if (with0) wave_bar(3, kWaveThreads);
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       if (nx.J != J) ob ^= 1;
       diag0 = with0;
