@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <thread>
 #include <vector>
@@ -215,6 +216,15 @@ struct RunOut {
   int sparse = 0;                   // polish sweeps run by the sparse polish
   int partial = 0;                  // screened sweeps that verified only their loud rows
 };
+
+// FP32 where the wave form runs: a screened sweep with more correction terms
+// than this per row is handed over, and screening resumes when a sweep changes
+// fewer pairs than that per row.  24-lambda paths to 0.08 (p, n), terms per
+// row 4000 / 2000 / 1000 / 500 / as many as fit the lists: (300, 300) 41 / 39 /
+// 39 / 40 / 131 ms, (500, 400) 48 / 46 / 47 / 49 / 100, (1000, 800) 57 / 58 /
+// 58 / 60 / 104, (1000, 3000) 17.6 / 17.5 / 18.8 / 20.6 / 19.2, (2000, 1000)
+// 134 / 138 / 138 / 144 / 186.
+constexpr int kDenseTermsPerRow = 3000, kDenseTermsMin = 1 << 19, kDenseResumePerRow = 12;
 
 // Whether the FP32 sweeps the screened kernel hands over take the wave form.
 bool dense_wave(concord_state* st) {
@@ -534,6 +544,8 @@ int launch_screened_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, d
   a.sdiag64 = st->sdiag64;
   a.omdiag64 = omdiag64;
   a.w = screen_work<T>(st);
+  if (sizeof(T) == 4 && dense_wave(st))
+    a.w.term_cap = std::min(a.w.term_cap, std::max(kDenseTermsPerRow * st->p, kDenseTermsMin));
   a.barrier = st->barrier;
   a.wait.abort = st->abort_info;
   a.wait.info = st->abort_info + 1;
@@ -628,8 +640,9 @@ int launch_screened_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, d
 
 // Sweeps in the state's chosen variant.  Screened launches run until the
 // stopping rule, the sweep budget, or a sweep whose candidates overflow the
-// lists; such a sweep (and any following sweep that still changes more than
-// half the list capacity) runs on the dense kernel, then screening resumes.
+// lists (or are more than the wave form takes for a sweep); such a sweep (and
+// any following sweep that still changes many pairs) runs on the dense kernel,
+// then screening resumes.
 template <typename T>
 int launch_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* omdiag64, double lambda,
                double tol, int stop_rule, int n_sweeps, int kkt_only, int hist_offset, int stall_stop,
@@ -643,6 +656,9 @@ int launch_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* om
     return launch_dense<T>(st, S, W, Om, sdiagT, omdiag64, lambda, tol, stop_rule, n_sweeps,
                            kkt_only, hist_offset, stall_stop, out);
   int done = 0, first_delta = 0, redos = 0, dense = 0;
+  const double resume = sizeof(T) == 4 && dense_wave(st)
+                            ? std::min(0.5 * st->nc_cap, (double)kDenseResumePerRow * st->p)
+                            : 0.5 * st->nc_cap;
   RunOut o;
   for (;;) {
     int code = 0;
@@ -672,7 +688,7 @@ int launch_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* om
       }
       RunOut dq;
       rc = launch_dense<T>(st, S, W, Om, sdiagT, omdiag64, lambda, tol, stop_rule, n_sweeps - done, 0,
-                           hist_offset + done, 0, &dq, true, 0.5 * st->nc_cap);
+                           hist_offset + done, 0, &dq, true, resume);
       if (dq.first_delta && !first_delta) first_delta = done + dq.first_delta;
       done += dq.sweeps;
       dense += dq.sweeps;
@@ -686,7 +702,7 @@ int launch_run(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* om
         *out = o;
         return rc;
       }
-      if (dq.active < 0.5 * st->nc_cap) break;
+      if (dq.active < resume) break;
     }
   }
 }
