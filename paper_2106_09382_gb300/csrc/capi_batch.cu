@@ -51,8 +51,13 @@ constexpr int kDenseRows = 8;  // dense layout of a screened batch that was not 
 // Candidate pairs and correction terms of a problem's screened sweeps; a
 // lambda that needs more runs on the dense kernel.  Smaller than a single
 // state's: a problem has a few SMs here, and its dense sweeps run beside the
-// other problems'.
+// other problems'.  FP32 lambdas that the wave form would take are handed over
+// sooner (candidates per row, at least, ms): 24 subsamples of p = 500, 8
+// lambdas to 0.3: 24, 16384: 20.3; 24, 4096: 16.2; 16, 4096: 12.3; 8, 2048:
+// 12.7; to 0.15: 50.9, 42.8, 45.9, 48.7; 32 of p = 200 to 0.2: 136, 39, 37,
+// 39; 8 of p = 1000: 35.6, 35.6, 38.2, 44.9.
 constexpr int kBatchCandPerRow = 24, kBatchCandMin = 16384, kBatchTermsPerCand = 32;
+constexpr int kBatchWaveCandPerRow = 16, kBatchWaveCandMin = 4096;
 
 // One problem's device arrays (T = float for CONCORD_MIXED, double for FP64).
 struct Prob {
@@ -380,7 +385,9 @@ int run_waves(concord_batch* bt, int rows, const std::vector<Item>& items,
 int ensure_screen(concord_batch* bt, Prob& q) {
   if (q.scr) return CONCORD_OK;
   const long long pairs = (long long)q.p * (q.p - 1) / 2;
-  long long nc = std::max((long long)kBatchCandPerRow * q.p, (long long)kBatchCandMin);
+  const bool wave = is_mixed(bt) && sweep_wave_blocks(q.p) <= std::min(kWaveMaxBlocks, bt->sms);
+  long long nc = wave ? std::max(kBatchWaveCandPerRow * q.p, kBatchWaveCandMin)
+                      : std::max(kBatchCandPerRow * q.p, kBatchCandMin);
   nc = std::max(1ll, std::min(nc, pairs));
   q.nc = (int)nc;
   q.tc = (int)std::min(nc * kBatchTermsPerCand, 1ll << 25);
