@@ -1444,8 +1444,10 @@ __device__ __forceinline__ void screened_body(const ScreenArgs<T>& a, const int 
                       // not captured: every change so far precedes the pair's step
                       if (!cap[uu][e]) vv[uu][e] = acc[uu][e];
                       out[e] = (last && dd != (T)0) ? fma_t(dd, si[uu][e], acc[uu][e]) : acc[uu][e];
-                      if (full && c_last < cx[uu][e]) vrow[e] = vv[uu][e];
+                      if (full && c_last >= 0 && c_last < cx[uu][e]) vrow[e] = vv[uu][e];
                     }
+                    // (the row's first changes: nothing is stored yet, whole vectors)
+                    if (full && c_last < 0) *reinterpret_cast<VV*>(vrow) = VT::join(vv[uu]);
                     reinterpret_cast<VV*>(Wn + (size_t)i * ld)[q] = VT::join(out);
                   }
                 }
