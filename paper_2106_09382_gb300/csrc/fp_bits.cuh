@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstring>
 
 namespace concord {
@@ -88,6 +89,52 @@ __host__ __device__ __forceinline__ float narrow_f64(double d) {
 // isfinite on the bit pattern (exponent field not all ones), integer only.
 __host__ __device__ __forceinline__ bool finite_bits(double v) {
   return ((fb_d2u(v) >> 52) & 0x7ffu) != 0x7ffu;
+}
+
+// (x - mean) * inv, each rounded to FP64, then rounded to FP32: the FP64 pipe
+// issues a warp's operation over 16 cycles, so the value is formed from pairs
+// of floats (difference and product with their rounding errors; Knuth's
+// two-sum, the product's error by an FMA), with a bound on all that is
+// dropped.  Where both ends of the bound round to the same float that float is
+// the result; elsewhere (2^-18 of all values; zeros, and the ends of the
+// range) the FP64 operations decide.  Bit-identical to them.
+__host__ __device__ __forceinline__ float fb_mul(float a, float b) {  // (never fused with a sum)
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+struct StdCol {
+  double mean, inv;
+  float mh, ml, ih, il;  // mean and inv as pairs
+};
+__host__ __device__ __forceinline__ StdCol std_col(double mean, double inv) {
+  StdCol c;
+  c.mean = mean;
+  c.inv = inv;
+  c.mh = narrow_f64(mean);
+  c.ml = narrow_f64(mean - to_f64(c.mh));
+  c.ih = narrow_f64(inv);
+  c.il = narrow_f64(inv - to_f64(c.ih));
+  // (a pair needs room below it: a NaN leaves every value to the FP64 path)
+  if (!(fabsf(c.ih) > 0x1p-60f && fabsf(c.ih) < 0x1p60f)) c.ih = NAN;
+  return c;
+}
+__host__ __device__ __forceinline__ float std_value(float x, const StdCol& c) {
+  const float s = x - c.mh;
+  const float t = s - x;
+  const float e = ((x - (s - t)) - (c.mh + t)) - c.ml;  // x - mean - s
+  const float p = fb_mul(s, c.ih);
+  const float q = fmaf(e, c.ih, fmaf(s, c.il, fmaf(s, c.ih, -p)));
+  // dropped: less than 2^-44 (|s| + |mean|) |inv|
+  const float bound = fb_mul(0x1p-42f, fb_mul(fabsf(s) + fabsf(c.mh), fabsf(c.ih)));
+  const float z0 = p + (q - bound), z1 = p + (q + bound);
+  if (z0 == z1 && fabsf(z0) > 0x1p-60f && fabsf(z0) < 0x1p60f && bound > 0x1p-100f) return z0;
+  return narrow_f64((to_f64(x) - c.mean) * c.inv);
+}
+__host__ __device__ __forceinline__ float std_value(double x, const StdCol& c) {
+  return narrow_f64((x - c.mean) * c.inv);
 }
 
 }  // namespace concord
