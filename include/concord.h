@@ -68,7 +68,9 @@ extern "C" {
 #define CONCORD_PREP_STANDARDIZE 2
 
 /* Gram arithmetic. */
-#define CONCORD_GRAM_FP64 0    /* FP64 CUDA-core products, FP64 accumulation */
+#define CONCORD_GRAM_FP64 0    /* FP64: exact digit products on the tensor cores summed as 64-bit
+                                  integers; FP64 CUDA cores where the digits do not resolve a
+                                  column and below 32 rows */
 #define CONCORD_GRAM_FP32 1    /* FP32 CUDA-core products, FP32 accumulation */
 #define CONCORD_GRAM_TF32X3 2  /* tensor cores (tcgen05, kind::tf32): each FP32
                                   operand split hi + lo, hi*hi + hi*lo + lo*hi,
