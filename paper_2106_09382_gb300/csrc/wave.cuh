@@ -100,6 +100,7 @@ struct WaveSmem {
   float e[NM][kWaveB], z[NM][kWaveB];      // W_I,0 and W_0,I of a diagonal tile
   float dd[NM][kWaveB];                    // diagonal changes
   unsigned need[2][NM][4];                 // j / 2 with changes [tile parity][m][half of rows, row parity]
+  float nw0[NM][kWaveB];                   // new values of the pairs (0, i)
   float s00[NM], sd0[NM];
   WaveArgs<NM> args;                       // (in registers they would be held through the sweep)
 };
@@ -538,8 +539,7 @@ __device__ __forceinline__ void wave_chain(int p, WaveSmem<NM>& s, Ops& ops, int
 // lanes hold as well.
 template <int NM, class Ops>
 __device__ __forceinline__ void wave_chain_diag(const WaveArgs<NM>& a, WaveSmem<NM>& s, Ops& ops, int i0,
-                                                int hl, int ll, bool with0, int db, int ob,
-                                                unsigned long long* zw, int nb, int lane) {
+                                                int hl, int ll, bool with0, int db, int ob, int lane) {
   constexpr unsigned FULL = 0xffffffffu;
   const int p = a.p, i = i0 + lane;
   const bool iok = i >= 1 && i < p;
@@ -593,15 +593,18 @@ __device__ __forceinline__ void wave_chain_diag(const WaveArgs<NM>& a, WaveSmem<
         s.om[ob][m][lane][r] = nw[m];
         need[m] |= d[m] != 0.f ? 1u << (r >> 1) : 0u;
       }
-      if (on && self) {
+      if (on && self) {  // (to memory and the other blocks after the steps)
         s.d0[db][m][lane] = d[m];
-        if (d[m] != 0.f) a.Om[m][(size_t)i * a.ld] = a.Om[m][i] = nw[m];
-        st_relaxed_u64(zw + (size_t)m * kWaveB * nb + i, wave_word(a.tag, d[m]));
+        s.nw0[m][lane] = nw[m];
       }
     }
     ops.count(d);
-    if (on && self) ops.count(d);  // vertex 0's row
-    __syncwarp();
+    if (with0) {  // vertex 0's row
+      float d0[NM];
+#pragma unroll
+      for (int m = 0; m < NM; ++m) d0[m] = self ? d[m] : 0.f;
+      ops.count(d0);
+    }
     const int vz = (sl >> 1) & 31;
     const bool zon = with0 && (sl & ~63) == 0;
 #pragma unroll
@@ -869,7 +872,7 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
       if (with0) wave_bar(3, kWaveThreads);
       wave_bar(1, kWaveFirst);
       if (I == J && wid == 0)
-        wave_chain_diag<NM>(a, s, ops, i0, t.hi - i0 - j0, t.lo - i0 - j0, with0, v & 1, ob, zw, nb, lane);
+        wave_chain_diag<NM>(a, s, ops, i0, t.hi - i0 - j0, t.lo - i0 - j0, with0, v & 1, ob, lane);
       else if (I != J)
         wave_chain<NM>(p, s, ops, i0, j0, t.hi - i0 - j0, t.lo - i0 - j0, v & 1, v & 1, ob, lane, wid);
       wave_bar(2, kWaveFirst);  // the tile's changes are in s.d
@@ -948,6 +951,14 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
         }
         if (nx.J != I) publish(nx, A);
       }
+      if (with0 && fw == 0 && 2 * lane >= t.lo - i0 - j0 && 2 * lane <= hl && i0 + lane >= 1 && i0 + lane < p)
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {  // vertex 0's pairs: to its row's holders, and to memory
+          const float d = s.d0[db][m][lane];
+          st_relaxed_u64(zw + (size_t)m * kWaveB * nb + i0 + lane, wave_word(a.tag, d));
+          if (d != 0.f)
+            a.Om[m][(size_t)(i0 + lane) * ld] = a.Om[m][i0 + lane] = s.nw0[m][lane];
+        }
 #pragma unroll
       for (int m = 0; m < NM; ++m)  // (column 0 is kept by vertex 0's pairs)
         if ((s.need[db][m][0] | s.need[db][m][1] | s.need[db][m][2] | s.need[db][m][3]) != 0) {
