@@ -543,39 +543,48 @@ __device__ __forceinline__ void wave_chain_diag(const WaveArgs<NM>& a, WaveSmem<
   constexpr unsigned FULL = 0xffffffffu;
   const int p = a.p, i = i0 + lane;
   const bool iok = i >= 1 && i < p;
-  float x[NM][16], e[NM], z[NM];
+  constexpr int KD = 2 * NM - 1;
+  float x[NM][16], e[NM], z[NM], sdl[NM], om[NM], c[NM], rc[KD];
   unsigned need[NM];
 #pragma unroll
   for (int m = 0; m < NM; ++m) {
     wave_row(x[m], s.a[m][lane]);
     e[m] = with0 ? s.e[m][lane] : 0.f;
     z[m] = with0 ? s.z[m][lane] : 0.f;
+    sdl[m] = s.sdi[m][lane];
     need[m] = 0;
     if (with0) s.d0[db][m][lane] = 0.f;
   }
+  // what the step with sum sl needs and does not wait for
+  auto operands = [&](int sl) {
+    const int rm = (sl - lane) & 31;
+    const bool self = sl - lane == lane;
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      om[m] = *(self ? &s.om0[m][lane] : &s.om[ob][m][lane][rm]);
+      c[m] = sdl[m] + *(self ? &s.sd0[m] : &s.sdi[m][rm]);
+    }
+#pragma unroll
+    for (int k = 0; k < KD; ++k) rc[k] = *(self ? &s.rz[k][lane] : &s.rc[db][k][lane][rm]);
+  };
+  operands(hl);
 #pragma unroll 1
   for (int sl = hl; sl >= ll; sl -= 2) {
     const int r = sl - lane, rm = r & 31;
     const bool self = r == lane;  // even sums: with0
     const int j = self ? 0 : i0 + r;
     const bool on = iok && r == rm && (self || (j >= 1 && j < p));
-    float wp[NM], d[NM];
+    float d[NM], wa[NM], wb[NM], n[NM], dn[NM], y[NM], nw[NM], o[NM];
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
-      wp[m] = __shfl_sync(FULL, x[m][0], rm);
-    }
-    float wa[NM], wb[NM], om[NM], c[NM], rc[2 * NM - 1], n[NM], dn[NM], y[NM], nw[NM];
-#pragma unroll
-    for (int k = 0; k < 2 * NM - 1; ++k) rc[k] = self ? s.rz[k][lane] : s.rc[db][k][lane][rm];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      const float wu = self ? e[m] : x[m][0], wv = self ? z[m] : wp[m];
+      const float wp = __shfl_sync(FULL, x[m][0], rm);
+      const float wu = self ? e[m] : x[m][0], wv = self ? z[m] : wp;
       wa[m] = i < j ? wu : wv;
       wb[m] = i < j ? wv : wu;
-      om[m] = self ? s.om0[m][lane] : s.om[ob][m][lane][rm];
-      c[m] = s.sdi[m][lane] + (self ? s.sd0[m] : s.sdi[m][rm]);
+      o[m] = om[m];
     }
     ops.pair(c, rc, om, wa, wb, n, dn, y);
+    operands(sl - 2);
     bool plain = true;
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
@@ -587,7 +596,7 @@ __device__ __forceinline__ void wave_chain_diag(const WaveArgs<NM>& a, WaveSmem<
       for (int m = 0; m < NM; ++m) nw[m] = n[m] != 0.f ? n[m] / dn[m] : 0.f;
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
-      d[m] = on ? nw[m] - om[m] : 0.f;
+      d[m] = on ? nw[m] - o[m] : 0.f;
       if (on && !self) {
         s.d[db][m][lane & 1][r >> 1][lane >> 1] = d[m];
         s.om[ob][m][lane][r] = nw[m];
@@ -675,19 +684,6 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
         wave_load(s.sjn[tb][m], a.S[m], j0, n0, p, ld, rt, kWaveRest);
         if (Jq >= 0) wave_load(s.spn[tb][m], a.S[m], kWaveB * Jq, n0, p, ld, rt, kWaveRest);
       }
-      if (m == 0)
-        for (int e = rt; e < kWaveB * kWaveB; e += kWaveRest) {
-          const int i = i0 + e / kWaveB, j = j0 + e % kWaveB;
-          float c[NM], dn[2 * NM - 1];
-#pragma unroll
-          for (int k = 0; k < NM; ++k)
-            c[k] = i < p && j < p ? __ldg(a.sdiag[k] + (size_t)i * a.sd_stride) +
-                                        __ldg(a.sdiag[k] + (size_t)j * a.sd_stride)
-                                  : 1.f;
-          Ops::denominators(c, dn);
-#pragma unroll
-          for (int k = 0; k < 2 * NM - 1; ++k) (&s.rc[tb][k][0][0])[e] = 1.f / dn[k];
-        }
       if (rt < kWaveB) {
         if (j0 + rt < p)
           cp_async4(&s.sd[tb][m][rt], a.sdiag[m] + (size_t)(j0 + rt) * a.sd_stride);
@@ -697,6 +693,22 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // rest: the reciprocals tile t's pairs need (divisions: after what others wait for)
+  auto reciprocals = [&](const WaveTile& t, int tb) {
+    const int j0 = kWaveB * t.J;
+    for (int e = rt; e < kWaveB * kWaveB; e += kWaveRest) {
+      const int i = i0 + e / kWaveB, j = j0 + e % kWaveB;
+      float c[NM], dn[2 * NM - 1];
+#pragma unroll
+      for (int k = 0; k < NM; ++k)
+        c[k] = i < p && j < p ? __ldg(a.sdiag[k] + (size_t)i * a.sd_stride) +
+                                    __ldg(a.sdiag[k] + (size_t)j * a.sd_stride)
+                              : 1.f;
+      Ops::denominators(c, dn);
+#pragma unroll
+      for (int k = 0; k < 2 * NM - 1; ++k) (&s.rc[tb][k][0][0])[e] = 1.f / dn[k];
+    }
   };
   // front: a tile's entries to the partner ((row + column) parity picks two rows per lane)
   auto publish = [&](const WaveTile& t, const float (&y)[NM][4]) {
@@ -818,6 +830,7 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
   }
   if (rest) {
     fetch(t, -1, nx, 0, 0);
+    reciprocals(t, 0);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
   int zdone = nb;  // zwarp: the changes of vertex 0's pairs in blocks >= zdone are in Z
@@ -990,6 +1003,7 @@ __device__ __forceinline__ void wave_sweep(int I, int rank, int cl, Ops& ops) {
                       kWaveRestWarps, lane, with0);
       else if (with0)
         wave_arrive(3, kWaveThreads);
+      if (nx.J >= 0) reciprocals(nx, db ^ 1);
       if (zwarp && !with0)
         while (zdone > 0 && zdone - 1 != I && zapply(zdone - 1, false)) --zdone;
       asm volatile("cp.async.wait_group 0;" ::: "memory");
