@@ -395,6 +395,14 @@ __device__ __forceinline__ void wave_row(float (&x)[16], const float* row) {
   }
 }
 
+// x one step on, no change.
+__device__ __forceinline__ void wave_turn(float (&x)[16]) {
+  const float first = x[0];
+#pragma unroll
+  for (int u = 0; u < 15; ++u) x[u] = x[u + 1];
+  x[15] = first;
+}
+
 // n / d, y the correctly rounded 1 / d: a quotient and its residual, twice.
 // With y correctly rounded and the quotient within an ulp the last correction
 // rounds correctly (Markstein, "Computation of elementary functions on the
@@ -523,12 +531,7 @@ __device__ __forceinline__ void wave_chain(int p, WaveSmem<NM>& s, Ops& ops, int
       if (side == 0) ops.count(d);
     } else {
 #pragma unroll
-      for (int m = 0; m < NM; ++m) {
-        const float first = x[m][0];
-#pragma unroll
-        for (int u = 0; u < 15; ++u) x[m][u] = x[m][u + 1];
-        x[m][15] = first;
-      }
+      for (int m = 0; m < NM; ++m) wave_turn(x[m]);
     }
   }
   if (side == 0) wave_needs<NM>(s, need, db, lane);
@@ -585,44 +588,52 @@ __device__ __forceinline__ void wave_chain_diag(const WaveArgs<NM>& a, WaveSmem<
     }
     ops.pair(c, rc, om, wa, wb, n, dn, y);
     operands(sl - 2);
-    bool plain = true;
+    bool loud = false;
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      nw[m] = wave_quotient(n[m], dn[m], y[m]);
-      plain = plain && wave_plain(n[m], dn[m]);
-    }
-    if (__any_sync(FULL, on && !plain))
+    for (int m = 0; m < NM; ++m) loud = loud || n[m] != 0.f || o[m] != 0.f;
+    if (NM == 1 || __any_sync(FULL, loud && on)) {  // (as in wave_chain)
+      bool plain = true;
 #pragma unroll
-      for (int m = 0; m < NM; ++m) nw[m] = n[m] != 0.f ? n[m] / dn[m] : 0.f;
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      d[m] = on ? nw[m] - o[m] : 0.f;
-      if (on && !self) {
-        s.d[db][m][lane & 1][r >> 1][lane >> 1] = d[m];
-        s.om[ob][m][lane][r] = nw[m];
-        need[m] |= d[m] != 0.f ? 1u << (r >> 1) : 0u;
+      for (int m = 0; m < NM; ++m) {
+        nw[m] = wave_quotient(n[m], dn[m], y[m]);
+        plain = plain && wave_plain(n[m], dn[m]);
       }
-      if (on && self) {  // (to memory and the other blocks after the steps)
-        s.d0[db][m][lane] = d[m];
-        s.nw0[m][lane] = nw[m];
-      }
-    }
-    ops.count(d);
-    if (with0) {  // vertex 0's row
-      float d0[NM];
+      if (__any_sync(FULL, on && !plain))
 #pragma unroll
-      for (int m = 0; m < NM; ++m) d0[m] = self ? d[m] : 0.f;
-      ops.count(d0);
-    }
-    const int vz = (sl >> 1) & 31;
-    const bool zon = with0 && (sl & ~63) == 0;
+        for (int m = 0; m < NM; ++m) nw[m] = n[m] != 0.f ? n[m] / dn[m] : 0.f;
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      wave_step(x[m], d[m], self ? s.t0[m][lane] : s.ti[m][rm]);
-      if (zon) {
-        e[m] = fmaf(d[m], self ? s.s00[m] : s.si0[m][rm], e[m]);
-        z[m] = fmaf(__shfl_sync(FULL, d[m], vz), s.sii[m][vz][lane], z[m]);
+      for (int m = 0; m < NM; ++m) {
+        d[m] = on ? nw[m] - o[m] : 0.f;
+        if (on && !self) {
+          s.d[db][m][lane & 1][r >> 1][lane >> 1] = d[m];
+          s.om[ob][m][lane][r] = nw[m];
+          need[m] |= d[m] != 0.f ? 1u << (r >> 1) : 0u;
+        }
+        if (on && self) {  // (to memory and the other blocks after the steps)
+          s.d0[db][m][lane] = d[m];
+          s.nw0[m][lane] = nw[m];
+        }
       }
+      ops.count(d);
+      if (with0) {  // vertex 0's row
+        float d0[NM];
+#pragma unroll
+        for (int m = 0; m < NM; ++m) d0[m] = self ? d[m] : 0.f;
+        ops.count(d0);
+      }
+      const int vz = (sl >> 1) & 31;
+      const bool zon = with0 && (sl & ~63) == 0;
+#pragma unroll
+      for (int m = 0; m < NM; ++m) {
+        wave_step(x[m], d[m], self ? s.t0[m][lane] : s.ti[m][rm]);
+        if (zon) {
+          e[m] = fmaf(d[m], self ? s.s00[m] : s.si0[m][rm], e[m]);
+          z[m] = fmaf(__shfl_sync(FULL, d[m], vz), s.sii[m][vz][lane], z[m]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < NM; ++m) wave_turn(x[m]);
     }
   }
 #pragma unroll
