@@ -255,7 +255,7 @@ int launch_dense(concord_state* st, T* S, T* W, T* Om, const T* sdiagT, double* 
   const bool layout_set = own && (st->sweep_variant == CONCORD_SWEEP_GRID ||
                                   st->sweep_variant == CONCORD_SWEEP_CLUSTER);
   // bandwidth: sweeps handed over by the screened kernel change most pairs;
-  // in FP32 they take the wave form (p = 1000: 0.8 ms a sweep, 3.3 ms colour by
+  // in FP32 they take the wave form (p = 1000: 0.7 ms a sweep, 3.3 ms colour by
   // colour), else the grid layout with one row per warp (all SMs stream rows)
   const bool wave = bandwidth && mixed && !kkt_only && dense_wave(st);
   if (bandwidth && !wave) n_sweeps = 1;

@@ -171,7 +171,7 @@ int run_phase(concord_joint* jt, bool f32, double l1, double l2, double tol, int
     a.hist_len = hist_left > 0 ? hist_left : 0;
     a.result = jt->result;
     // the wave form unless the caller chose a grid or the barrier, or tests a
-    // failing row: p = 1000, 9 sweeps: 45 ms colour by colour, 10.7 ms
+    // failing row: p = 1000, 9 sweeps: 45 ms colour by colour, 7.5 ms
     const int blocks = joint_wave_blocks(jt->p);
     if (rv && jt->grid_override == 0 && fault_row < 0 && blocks <= kWaveMaxBlocks && blocks <= grid) {
       const size_t bytes = sizeof(unsigned long long) * joint_wave_words(jt->p);

@@ -27,10 +27,12 @@
 // 0's row is spread over the owners by columns; its changes are published as
 // words too.
 //
-// p = 1000, FP32, a tile of one matrix / two: 14.8 / 17.5 us, of which the
-// steps 7.8 / 7.1 us, the wait for the partner 4.7 / 7.3 us (tiles of a wave
-// differ); with sixteen warps walking the steps together behind a CTA barrier
-// and then updating everything 22 / 35 us.
+// p = 1000, FP32, a tile of one matrix: 9.9 us, of which the steps 5.5, the
+// wait for the partner 1.4, the next tile's columns and their publication 2.8;
+// with sixteen warps walking the steps together behind a CTA barrier and then
+// updating everything 22 us.  What bounds it is the chain: swap, pair, FMA of
+// a step (~0.17 us), and a diagonal tile's longer steps (7 - 8 us a tile).
+// 32-lambda path 293 -> 119 ms, joint solve of 9 sweeps 22.3 -> 8.2 ms.
 //
 // Every entry of W gets the same FMAs in the same order as in the colour-by-
 // colour kernels (a row's changes in step order), so the iterates are theirs
